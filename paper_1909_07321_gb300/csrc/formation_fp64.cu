@@ -3,39 +3,168 @@
 // (tri_idx, stride tri_ld(n)).
 //
 // This is the plain-FP64 baseline the mixed-precision path is measured
-// against. Only the upper triangle is computed (tiles with tile_j >= tile_i)
-// and stored, so every R is exactly symmetric. d_k = 1/(E_k - E) is formed
-// once per (tile, k) in shared memory and folded into the j-operand.
+// against. Only the upper triangle is computed and stored, so every R is
+// exactly symmetric. d_k = 1/(E_k - E) is formed once per (CTA, k) in shared
+// memory and folded into the j-operand.
 #include "rm_internal.cuh"
 
 namespace rmgb {
 namespace {
 
-// n < 32: one thread per (energy, i <= j), plain loop over poles.
-__global__ void form_r_naive(PwDev pw, const double *__restrict__ E, int nE,
-                             double *__restrict__ R)
+// n <= PK_MAX_N: the packed pairs p = (i <= j) of one energy dealt out 32 to a
+// warp load, PT loads a warp, so that no FP64 FMA is spent on an entry that is
+// not stored. GB300 issues 2 FP64 FMAs per clock and SM, and everything else
+// (two shared loads per FMA, the staging) fits beside them; a 64 x 64 tile
+// kernel spends 3072 FMAs per pole where 64 channels need 2080, and 21504
+// where 132 need 8778. 4000 energies of 64 channels x 1920 poles: 39.9 ms
+// tiled, 27.6 ms packed (floor 27.4); 200 of 132 x 3960: 30.4 and 13.1 ms
+// (floor 11.9).
+//
+// A CTA takes NW PT warp loads of one energy, from row rlo on: per chunk of TK
+// poles it stages the rows rlo .. n - 1 of W and of W d (DIV: W / (E_k - E),
+// n < 32) in shared memory (row stride TK + 1 doubles: lanes on consecutive
+// rows j read distinct banks), the next chunk's W and the chunk after that
+// one's d already on their way. Every entry is one chain of FMAs over
+// ascending poles.
+constexpr int PK_MAX_N = 1024;
+constexpr int PK_MAX_WARPS = 16;
+
+template <int PT, int TK, bool DIV>
+__global__ void __launch_bounds__(PK_MAX_WARPS * 32)
+    form_r_packed(PwDev pw, const double *__restrict__ E, double *__restrict__ R)
 {
-    const int n = pw.n;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)nE * n * n) return;
-    const int e = (int)(idx / ((long long)n * n));
-    const int ij = (int)(idx - (long long)e * n * n);
-    const int i = ij / n, j = ij - (ij / n) * n;
-    if (i > j) return;
-    const double x = E[e];
-    const double *wi = pw.W + (size_t)i * pw.N;
-    const double *wj = pw.W + (size_t)j * pw.N;
-    double acc = 0.0;
-    for (int k = 0; k < pw.N; ++k) acc = fma(wi[k], wj[k] / (pw.Ek[k] - x), acc);
-    acc *= 0.5 / pw.a;
-    R[(size_t)e * tri_ld(n) + tri_idx(i, j, n)] = acc;
+    extern __shared__ double sm[];
+    const int n = pw.n, N = pw.N, np = tri_count(n);
+    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const double x = E[blockIdx.y];
+    const int p_cta = blockIdx.x * nthr * PT;
+    auto row_of = [&](int p) {   // row of packed pair p
+        const float t = (float)(2 * n + 1);
+        int i = (int)((t - sqrtf(fmaxf(t * t - 8.0f * (float)p, 0.0f))) * 0.5f);
+        i = min(max(i, 0), n - 1);
+        while (i > 0 && tri_idx(i, i, n) > p) --i;
+        while (i + 1 < n && tri_idx(i + 1, i + 1, n) <= p) ++i;
+        return i;
+    };
+    const int rlo = row_of(p_cta), nr = n - rlo;
+    constexpr int LD = TK + 1;
+    double *Ws = sm, *Wd = sm + nr * LD, *dk = Wd + nr * LD;   // dk: [2][TK]
+    // offsets of the pairs' rows; past the end, those of the last pair
+    int io[PT], jo[PT];
+    double acc[PT];
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int p = min(p_cta + (warp * PT + q) * 32 + lane, np - 1);
+        const int i = row_of(p);
+        io[q] = (i - rlo) * LD;
+        jo[q] = (i + (p - tri_idx(i, i, n)) - rlo) * LD;
+        acc[q] = 0.0;
+    }
+    const int total = nr * TK;
+    const double *Wg = pw.W + (size_t)rlo * N;
+    auto den = [&](int k) { return k < N ? pw.Ek[k] - x : 1.0; };
+    if (tid < 2 * TK) dk[tid] = DIV ? den(tid) : (tid < N ? 1.0 / den(tid) : 0.0);
+    constexpr int PRE = 4;   // elements of the next chunk a thread holds
+    double pre[PRE];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+            const int q = tid + u * nthr, r = q / TK, c = q - r * TK;
+            pre[u] = q < total && k0 + c < N ? Wg[(size_t)r * N + k0 + c] : 0.0;
+        }
+    };
+    fetch(0);
+    __syncthreads();
+    for (int k0 = 0, b = 0; k0 < N; k0 += TK, b ^= 1) {
+        const double *dc = dk + b * TK;
+        auto put = [&](int q, double w) {
+            const int r = q / TK, c = q - r * TK;
+            Ws[r * LD + c] = w;
+            Wd[r * LD + c] = DIV ? w / dc[c] : w * dc[c];
+        };
+#pragma unroll
+        for (int u = 0; u < PRE; ++u)
+            if (tid + u * nthr < total) put(tid + u * nthr, pre[u]);
+        for (int q = tid + PRE * nthr; q < total; q += nthr) {
+            const int r = q / TK, c = q - r * TK;
+            put(q, k0 + c < N ? Wg[(size_t)r * N + k0 + c] : 0.0);
+        }
+        __syncthreads();
+        if (k0 + TK < N) fetch(k0 + TK);
+        if (tid < TK) {
+            const int k = k0 + 2 * TK + tid;
+            dk[b * TK + tid] = DIV ? den(k) : (k < N ? 1.0 / den(k) : 0.0);
+        }
+#pragma unroll
+        for (int c = 0; c < TK; ++c)
+#pragma unroll
+            for (int q = 0; q < PT; ++q) acc[q] = fma(Ws[io[q] + c], Wd[jo[q] + c], acc[q]);
+        __syncthreads();
+    }
+    const double h = 0.5 / pw.a;
+    double *Re = R + (size_t)blockIdx.y * tri_ld(n);
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int p = p_cta + (warp * PT + q) * 32 + lane;
+        if (p < np) Re[p] = acc[q] * h;
+    }
+}
+
+template <int PT, int TK, bool DIV>
+cudaError_t launch_packed(const PwDev &pw, const double *E, int nE, double *R, int nw, int ctas, cudaStream_t s)
+{
+    const size_t smem = ((size_t)2 * pw.n * (TK + 1) + 2 * TK) * sizeof(double);
+    const cudaError_t e = cudaFuncSetAttribute(form_r_packed<PT, TK, DIV>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    form_r_packed<PT, TK, DIV><<<dim3(ctas, nE), nw * 32, smem, s>>>(pw, E, R);
+    return cudaGetLastError();
+}
+
+// Loads per warp, warps and CTAs per energy: the least of CTAs x (warp-load
+// lanes + rows to be scaled), the FP64 work of a pole.
+cudaError_t launch_packed_any(const PwDev &pw, const double *E, int nE, double *R, cudaStream_t s)
+{
+    const int n = pw.n, nq = (tri_count(n) + 31) / 32;
+    int pt = 1, nw = 1, ctas = nq;
+    if (n < 32) {
+        pt = nq <= 4 ? 1 : (nq <= 8 ? 2 : 4);
+        nw = (nq + pt - 1) / pt;
+        ctas = 1;
+    } else {
+        long long best = 0;
+        for (int p = 4; p <= 8; ++p)
+            for (int w = 4; w <= PK_MAX_WARPS; ++w) {
+                const int c = (nq + p * w - 1) / (p * w);
+                const long long cost = (long long)c * (32 * p * w + n);
+                if (best == 0 || cost < best) {
+                    best = cost;
+                    pt = p;
+                    nw = w;
+                    ctas = c;
+                }
+            }
+    }
+#define RM_PK(P, K, D) launch_packed<P, K, D>(pw, E, nE, R, nw, ctas, s)
+    if (n < 32) return pt == 1 ? RM_PK(1, 16, true) : (pt == 2 ? RM_PK(2, 16, true) : RM_PK(4, 16, true));
+    // poles per chunk: at most ~70 KB of shared memory, three CTAs per SM
+#define RM_PK_TK(P) (n <= 256 ? RM_PK(P, 16, false) : (n <= 512 ? RM_PK(P, 8, false) : RM_PK(P, 4, false)))
+    switch (pt) {
+    case 4: return RM_PK_TK(4);
+    case 5: return RM_PK_TK(5);
+    case 6: return RM_PK_TK(6);
+    case 7: return RM_PK_TK(7);
+    default: return RM_PK_TK(8);
+    }
+#undef RM_PK_TK
+#undef RM_PK
 }
 
 constexpr int TB = 64;   // output tile
 constexpr int TK = 16;   // pole chunk
 constexpr int TT = 4;    // outputs per thread per dimension
 
-// n >= 32: CTA per (energy, 64x64 upper tile); 256 threads x 4x4 outputs.
+// n > PK_MAX_N: CTA per (energy, 64x64 upper tile); 256 threads x 4x4 outputs.
 // Off-diagonal tiles: thread (ty, tx) = (tid/16, tid%16) owns rows 4ty.., cols
 // 4tx... Diagonal tiles: the 32x32 quadrant below the diagonal is not needed,
 // so whole warps are assigned to the three upper quadrants (2 warps each) and
@@ -123,14 +252,10 @@ cudaError_t launch_form_r_fp64(const PwDev &pw, const double *E, int nE, double 
                                cudaStream_t s)
 {
     if (nE == 0) return cudaSuccess;
-    if (pw.n < 32) {
-        const long long total = (long long)nE * pw.n * pw.n;
-        form_r_naive<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(pw, E, nE, R);
-    } else {
-        const int t = (pw.n + TB - 1) / TB;
-        dim3 grid(t, t, nE);
-        form_r_tiled<<<grid, 256, 0, s>>>(pw, E, R);
-    }
+    if (pw.n <= PK_MAX_N) return launch_packed_any(pw, E, nE, R, s);
+    const int t = (pw.n + TB - 1) / TB;
+    dim3 grid(t, t, nE);
+    form_r_tiled<<<grid, 256, 0, s>>>(pw, E, R);
     return cudaGetLastError();
 }
 
