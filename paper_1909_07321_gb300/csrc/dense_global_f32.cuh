@@ -1,22 +1,23 @@
 // FP32 dense kernels of the global-memory solver's mixed-precision path
 // (rm_opts.solve_precision = RM_FP32, channel counts above the shared-memory
-// solver's limit). One CTA of 512 threads works on one energy's matrices in
+// solver's limit). One CTA (256 threads for the narrower systems, so that two
+// share an SM, 512 for the wider ones) works on one energy's matrices in
 // global memory:
 //
 //   lu32_factor_solve   [A | B] -> solves A X = B for the trailing rows of X
 //                       (the matching system, Section "Overview", Eq. match):
 //                       blocked right-looking LU with partial pivoting. The
 //                       current panel of PB columns (all rows below its
-//                       diagonal) is held in shared memory, column-major, and
-//                       factored there (two barriers per column: the row
-//                       update of one column carries the pivot search of the
-//                       next); its row interchanges are applied to the
+//                       diagonal) is factored with its rows in registers
+//                       (one barrier per column) and left in shared memory,
+//                       column-major; its row interchanges are applied to the
 //                       columns to its right as one permutation per panel;
 //                       U12 = L11^{-1} A12 is solved one column per thread;
 //                       the trailing matrix takes the rank-PB update
-//                       A22 -= L21 U12 in tiles of 128 x 128 with 4 x 8
-//                       register tiles per thread (the U12 strips staged in
-//                       two shared buffers in turn). Back-substitution of the
+//                       A22 -= L21 U12 in strips of 128 columns with 4 x 8
+//                       register tiles per thread, packed FMAs (the U12 strips
+//                       copied asynchronously into two shared buffers in
+//                       turn). Back-substitution of the
 //                       requested rows runs in the same blocked form, upwards.
 //   zsweep_invert       Z <- -Z^{-1} for a complex symmetric Z whose
 //                       Hermitian part is positive definite (Z = 1 - iK, the
@@ -27,11 +28,22 @@
 //                       shared memory (B -> -B^{-1}), the panel
 //                       P = Z[:, K] B^{-1} is formed in shared memory, every
 //                       other entry takes Z_ij -= P_i Z_Kj (rank-PB complex
-//                       update in tiles of 128 x 64, 4 x 4 per thread), and
+//                       update in strips of 64 columns, 4 x 4 per thread,
+//                       packed FMAs), and
 //                       Z[:, K], Z[K, :] become P and P^T. Z stays symmetric,
 //                       so only the upper triangle is kept current: tiles
 //                       wholly below the diagonal are skipped and every read
 //                       takes the entry (min(i, j), max(i, j)).
+//
+// At 1000 channels both stream their trailing matrix through HBM once per
+// panel (152 CTAs hold 1.2 GB) and are bound by that; below about 300 they
+// were bound by the latency of the panel's columns, which the registers and
+// the second CTA per SM take away. ms for 304 or more systems filling the GPU,
+// before and after: LU of 110 unknowns (1216 systems) 1.61 -> 0.46, 203 (912)
+// 2.85 -> 1.11, 431 (456) 5.37 -> 3.44, 1000 (304, 600 right-hand sides) 22.1
+// -> 19.1; sweep of 80 (1216) 0.63 -> 0.39, 150 (912) 1.38 -> 1.00, 300 (456)
+// 2.79 -> 2.30, 600 (304) 11.5 -> 11.0. Every entry keeps its chain of FMAs,
+// so the results are the same to the bit.
 //
 // Both kernels read and write their matrix through global memory (L2), with
 // no waits other than __syncthreads. A zero or non-finite pivot marks the
@@ -45,10 +57,9 @@
 namespace rmgb {
 namespace f32d {
 
-constexpr int NTH = 512;
-constexpr int NWARP = NTH / 32;
 constexpr int UW = 128;    // real strip width (columns)
 constexpr int UWC = 64;    // complex strip width (columns)
+constexpr int LU_SLOT = 36;   // floats of one warp's pivot candidate: its row (32), key, position
 
 // Layout of the real augmented matrix of n unknowns and np right-hand sides:
 // columns [0, n) A, [n, rhs0(n)) zero, [rhs0(n), rhs0(n) + np) B, zero up to ld.
@@ -61,18 +72,55 @@ __host__ __device__ inline int lu_npad(int n) { return ((rhs0(n) + 31) & ~31) + 
 __host__ __device__ inline int z_ld(int m) { return (m + 3) & ~3; }
 __host__ __device__ inline int z_npad(int m) { return ((m + 7) & ~7) + 8; }
 
-template <int PB> __host__ __device__ inline size_t lu_smem(int n)
+template <int PB, int NTH, int RPT> __host__ __device__ inline size_t lu_smem(int n)
 {
-    const size_t f = (size_t)PB * lu_npad(n) + 2 * (size_t)PB * (UW + 4);
+    const size_t f = (size_t)PB * lu_npad(n) + 2 * (size_t)PB * (UW + 4) + (RPT > 0 ? 2 * (NTH / 32) * LU_SLOT : 0);
     // perm [npad], move lists [2 PB], counters [8], reduction keys
     // [NWARP x 64 bit], reduction values [NWARP], and slack
-    const size_t i = (size_t)lu_npad(n) + 2 * PB + 8 + 3 * NWARP + 16;
+    const size_t i = (size_t)lu_npad(n) + 2 * PB + 8 + 3 * (NTH / 32) + 16;
     return f * sizeof(float) + i * sizeof(int);
 }
 
-template <int PB> __host__ __device__ inline size_t z_smem(int m)
+// LEAN: one strip, and operand pairs formed at each use instead of stored
+// (the widest systems whose panel of PB columns still fits).
+template <int PB, bool LEAN> __host__ __device__ inline size_t z_smem(int m)
 {
-    return ((size_t)PB * z_npad(m) + (size_t)PB * (UWC + 2) + (size_t)PB * (PB + 1)) * sizeof(float2);
+    const size_t panel = (size_t)PB * z_npad(m) * sizeof(float2), block = (size_t)PB * (PB + 1) * sizeof(float2);
+    if (LEAN) return panel + (size_t)PB * (UWC + 2) * sizeof(float2) + block;
+    return panel + 2 * (size_t)PB * (UWC + 2) * sizeof(float4) + (size_t)PB * PB * sizeof(float4) + block;
+}
+
+// Packed FP32 FMA: each half is fma(a, b, c) of that half, rounded as the
+// scalar instruction rounds it. The FMA pipe takes two clocks for it, so the
+// rank updates run at the pipe's rate with half the issue slots.
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack2(float x, float y)
+{
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int bytes = in ? 16 : 0;   // 0: the 16 bytes are zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
 // Packed key of a pivot candidate: larger magnitude first, then lower row.
@@ -97,211 +145,332 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long k)
 
 // ---- real blocked LU ---------------------------------------------------------
 
-// C[rows, cols c0..c0+128) -= Lp[0..PB)[rows] * Us[0..PB)[cols] for rows
-// [rlo, rhi), stored only where row in [rstore, rhi) and col < ld. Lp is the
-// column-major panel (stride npad), Us the staged strip (stride UW + 4).
-// Thread (ty, tx) = (tid / 16, tid % 16) takes rows 4 ty .. 4 ty + 3 of each
-// 128-row tile and columns 4 tx .. 4 tx + 3 and 64 + 4 tx .. 64 + 4 tx + 3
-// (a quarter-warp's float4 reads of Us hit distinct banks).
-template <int PB>
-__device__ __forceinline__ void lu_update_strip(float *M, int ld, int rlo, int rhi, int rstore, int c0,
-                                                const float *Lp, int npad, const float *Us)
+// Rows [rlo, rhi) (stored from rstore; rlo a multiple of 4), columns
+// [c_lo, w): C += Lp x U, Lp the column-major panel of PB columns (stride
+// npad) holding the negated multipliers, U = rows [u0, u0 + PB) of M (final,
+// zero from column w to ld). Strips of 128 columns, their U copied
+// asynchronously into two shared buffers in turn (one barrier per strip);
+// thread (ty, tx) = (tid / 16, tid % 16) takes rows 4 ty .. 4 ty + 3 of each
+// tile of NTH / 4 rows and columns 4 tx .. 4 tx + 3 and 64 + 4 tx .. 64 + 4 tx
+// + 3 (a quarter-warp's float4 reads of U hit distinct banks). The C tile
+// after the current one, the next strip's first at a strip's end, is on its
+// way into registers while one is updated.
+template <int PB, int NTH>
+__device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int rstore, int c_lo, int w, const float *Lp,
+                               int npad, float *Us)
 {
+    constexpr int TR = NTH / 4;   // rows per tile
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int cb[2] = {c0 + 4 * tx, c0 + 64 + 4 * tx};
-    // C tile of rows rb .. rb + 3 into v (zero outside [rstore, rhi) or past ld)
-    auto load = [&](int rb, float (&v)[4][8]) {
+    const int nstrip = (w - c_lo + UW - 1) / UW;
+    auto stage = [&](int s, float *buf) {
+        for (int q = tid; q < PB * (UW / 4); q += NTH) {
+            const int k = q / (UW / 4), j4 = 4 * (q - (q / (UW / 4)) * (UW / 4));
+            const int c = c_lo + s * UW + j4;
+            cp_async16(buf + k * (UW + 4) + j4, M + (size_t)(u0 + k) * ld + min(c, ld - 4), c < ld);
+        }
+    };
+    auto load = [&](int rb, int c0, unsigned long long (&v)[4][4]) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int r = rb + i;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (r < rhi && r >= rstore && cb[h] < ld)
-                    q = *reinterpret_cast<const float4 *>(M + (size_t)r * ld + cb[h]);
-                v[i][4 * h + 0] = q.x;
-                v[i][4 * h + 1] = q.y;
-                v[i][4 * h + 2] = q.z;
-                v[i][4 * h + 3] = q.w;
+                const int c = c0 + 64 * h + 4 * tx;
+                ulonglong2 q = make_ulonglong2(0ull, 0ull);
+                if (r < rhi && r >= rstore && c < ld) q = *reinterpret_cast<const ulonglong2 *>(M + (size_t)r * ld + c);
+                v[i][2 * h] = q.x;
+                v[i][2 * h + 1] = q.y;
             }
-        }
-    };
-    // the next row tile's C is loaded while this one is updated
-    float acc[4][8], nxt[4][8];
-    int rb = rlo + ty * 4;
-    if (rb < rhi) load(rb, acc);
-    for (int r0 = rlo; r0 < rhi; r0 += 128, rb += 128) {
-        if (rb >= rhi) break;
-        if (rb + 128 < rhi) load(rb + 128, nxt);
-        const bool full = rb + 3 < rhi;
-#pragma unroll 4
-        for (int k = 0; k < PB; ++k) {
-            float a[4], b[8];
-            if (full) {
-                const float4 a0 = *reinterpret_cast<const float4 *>(Lp + k * npad + rb);
-                a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = (rb + i < rhi) ? Lp[k * npad + rb + i] : 0.f;
-            }
-            const float4 b0 = *reinterpret_cast<const float4 *>(Us + k * (UW + 4) + 4 * tx);
-            const float4 b1 = *reinterpret_cast<const float4 *>(Us + k * (UW + 4) + 64 + 4 * tx);
-            b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
-            b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(-a[i], b[j], acc[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = rb + i;
-            if (r >= rhi || r < rstore) continue;
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if (cb[h] < ld)
-                    *reinterpret_cast<float4 *>(M + (size_t)r * ld + cb[h]) =
-                        make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = nxt[i][j];
-    }
-}
-
-// Rows [rlo, rhi) (stored from rstore), columns [c_lo, w): C -= Lp[0..PB) x
-// U, where U = rows [u0, u0 + PB) of M (final). Strips of 128 columns, their
-// U staged in two shared buffers in turn (one barrier per strip).
-template <int PB>
-__device__ void lu_update_rows(float *M, int ld, int u0, int kb, int rlo, int rhi, int rstore, int c_lo, int w,
-                               const float *Lp, int npad, float *Us)
-{
-    const int tid = threadIdx.x;
-    const int nstrip = (w - c_lo + UW - 1) / UW;
-    auto stage = [&](int s, float *buf) {
-        const int c0 = c_lo + s * UW;
-        for (int q = tid; q < PB * UW; q += NTH) {
-            const int k = q / UW, jj = q - (q / UW) * UW;
-            const int c = c0 + jj;
-            buf[k * (UW + 4) + jj] = (k < kb && c < w) ? M[(size_t)(u0 + k) * ld + c] : 0.f;
         }
     };
     stage(0, Us);
-    __syncthreads();
+    unsigned long long acc[4][4], nxt[4][4];
+    const int rb0 = rlo + 4 * ty;
+    load(rb0, c_lo, acc);
     for (int s = 0; s < nstrip; ++s) {
-        float *cur = Us + (s & 1) * PB * (UW + 4);
-        if (s + 1 < nstrip) stage(s + 1, Us + ((s + 1) & 1) * PB * (UW + 4));
-        lu_update_strip<PB>(M, ld, rlo, rhi, rstore, c_lo + s * UW, Lp, npad, cur);
+        const float *cur = Us + (s & 1) * PB * (UW + 4);
+        const int c0 = c_lo + s * UW;
+        cp_async_wait();
         __syncthreads();
+        if (s + 1 < nstrip) stage(s + 1, Us + ((s + 1) & 1) * PB * (UW + 4));
+        int rb = rb0;
+        for (int r0 = rlo; r0 < rhi; r0 += TR, rb += TR) {
+            const bool last = r0 + TR >= rhi;
+            if (!last) load(rb + TR, c0, nxt);
+            else if (s + 1 < nstrip) load(rb0, c0 + UW, nxt);
+            if (rb < rhi) {   // reads of Lp past rhi stay within the panel and feed rows that are not stored
+#pragma unroll 4
+                for (int k = 0; k < PB; ++k) {
+                    const float4 a4 = *reinterpret_cast<const float4 *>(Lp + k * npad + rb);
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(cur + k * (UW + 4) + 4 * tx);
+                    const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(cur + k * (UW + 4) + 64 + 4 * tx);
+                    const unsigned long long a[4] = {pack2(a4.x, a4.x), pack2(a4.y, a4.y), pack2(a4.z, a4.z),
+                                                     pack2(a4.w, a4.w)};
+                    const unsigned long long b[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(a[i], b[j], acc[i][j]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = rb + i;
+                    if (r >= rhi || r < rstore) continue;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int c = c0 + 64 * h + 4 * tx;
+                        if (c < ld)
+                            *reinterpret_cast<ulonglong2 *>(M + (size_t)r * ld + c) =
+                                make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = nxt[i][j];
+        }
     }
+    __syncthreads();
 }
 
-// Solves A X = B in place for the n x w augmented matrix M (row stride ld,
-// A in columns [0, n), right-hand sides in [rhs, w), zero padding between and
-// after), leaving X in rows [row_lo, n) of the right-hand-side columns.
-// Returns false if a pivot is zero or not finite.
-template <int PB>
-__device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int row_lo, float *smem)
+// Factors the panel of columns [k0, k0 + kb), rows [k0, n), with partial
+// pivoting (largest magnitude, then lowest row). On return Lp[j][r] holds the
+// factored panel in its final row order, entries below the diagonal negated,
+// and perm[r] the row that position r came from. A thread keeps RPT rows of
+// the panel in registers, so a column costs one barrier: every warp puts its
+// candidate (the row itself, key and position) into a slot before it, and all
+// take the best slot after it; rows change position only in a register.
+// Measured with the panel's rows in shared memory and two barriers: 2300 (203
+// rows) to 2900 (1000 rows) clocks a column.
+template <int PB, int NTH, int RPT>
+__device__ bool lu_panel_regs(const float *M, int ld, int n, int k0, int kb, float *Lp, int npad, int *perm, float *slots)
 {
+    constexpr int NW = NTH / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int npad = lu_npad(n);
-    float *Lp = smem;
-    float *Us = Lp + (size_t)PB * npad;
-    int *perm = reinterpret_cast<int *>(Us + 2 * PB * (UW + 4));
-    int *mv_dst = perm + npad;
-    int *mv_src = mv_dst + PB;
-    int *sh_int = mv_src + PB;                 // [0]: move count, [1]: bad
-    unsigned long long *red = reinterpret_cast<unsigned long long *>(sh_int + 8);   // [NWARP]
-    float *red_val = reinterpret_cast<float *>(red + NWARP);                        // [NWARP]
-
-    for (int k0 = 0; k0 < n; k0 += PB) {
-        const int kb = min(PB, n - k0);
-        // panel rows [k0, n), columns [k0, k0 + kb) -> Lp[j][r]
-        for (int q = tid; q < (n - k0) * kb; q += NTH) {
-            const int r = k0 + q / kb, j = q - (q / kb) * kb;
-            Lp[j * npad + r] = M[(size_t)r * ld + k0 + j];
+    float a[RPT][PB];
+    int pos[RPT];
+    bool live[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = k0 + tid + q * NTH;
+        pos[q] = r;
+        live[q] = r < n;
+#pragma unroll
+        for (int g = 0; g < PB; g += 4) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r < n && k0 + g < ld) v = *reinterpret_cast<const float4 *>(M + (size_t)r * ld + k0 + g);
+            a[q][g] = v.x;
+            a[q][g + 1] = v.y;
+            a[q][g + 2] = v.z;
+            a[q][g + 3] = v.w;
         }
-        for (int r = k0 + tid; r < n; r += NTH) perm[r] = r;
-        if (tid == 0) sh_int[0] = 0;
+    }
+#pragma unroll
+    for (int j = 0; j < PB; ++j) {
+        if (j >= kb) break;
+        const int c = k0 + j;
+        float *slot = slots + (j & 1) * NW * LU_SLOT;
+        // key 0: no row left; a NaN counts as infinity (and is then not finite)
+        unsigned mag = 0u;
+        int mp = 0x7fffffff, mq = 0;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            unsigned u = __float_as_uint(fabsf(a[q][j]));
+            u = u > 0x7f800000u ? 0x7f800000u : u;
+            if (live[q] && (mp == 0x7fffffff || u > mag || (u == mag && pos[q] < mp))) {
+                mag = u;
+                mp = pos[q];
+                mq = q;
+            }
+        }
+        const unsigned wm = __reduce_max_sync(0xffffffffu, mag);
+        const unsigned wp = __reduce_min_sync(0xffffffffu, mag == wm ? (unsigned)mp : 0x7fffffffu);
+        if (mag == wm && (unsigned)mp == wp && wp != 0x7fffffffu) {
+            float *dst = slot + warp * LU_SLOT;
+#pragma unroll
+            for (int q = 0; q < RPT; ++q)
+                if (mq == q) {
+#pragma unroll
+                    for (int g = (j & ~3); g < PB; g += 4)
+                        *reinterpret_cast<float4 *>(dst + g) = make_float4(a[q][g], a[q][g + 1], a[q][g + 2], a[q][g + 3]);
+                }
+            *reinterpret_cast<float2 *>(dst + PB) = make_float2(__uint_as_float(wm), __int_as_float((int)wp));
+        } else if (lane == 0 && wp == 0x7fffffffu) {
+            *reinterpret_cast<float2 *>(slot + warp * LU_SLOT + PB) = make_float2(0.f, __int_as_float(0x7fffffff));
+        }
         __syncthreads();
-        // pivot candidates of the panel's first column
-        {
-            unsigned long long key = 0ull;
-            float kv = 0.f;
-            for (int r = k0 + tid; r < n; r += NTH) {
-                const float v = Lp[r];
+        float2 cand = make_float2(0.f, __int_as_float(0x7fffffff));
+        if (lane < NW) cand = *reinterpret_cast<const float2 *>(slot + lane * LU_SLOT + PB);
+        const unsigned cm = __float_as_uint(cand.x), cp = (unsigned)__float_as_int(cand.y);
+        const unsigned bm = __reduce_max_sync(0xffffffffu, cm);
+        const unsigned p = __reduce_min_sync(0xffffffffu, cm == bm ? cp : 0x7fffffffu);
+        const int win = __ffs(__ballot_sync(0xffffffffu, cm == bm && cp == p)) - 1;
+        const float *pr = slot + win * LU_SLOT;
+        const float pv = pr[j];
+        if (!(fabsf(pv) > 0.f) || !isfinite(pv)) return false;   // the same decision in every thread
+        const float ipv = 1.0f / pv;
+        float l[RPT];   // 0 for rows already placed: they keep their entries
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            l[q] = 0.f;
+            if (live[q]) {
+                if (pos[q] == (int)p) {
+                    live[q] = false;
+                    pos[q] = c;
+                } else {
+                    if (pos[q] == c) pos[q] = (int)p;
+                    l[q] = a[q][j] * ipv;
+                    a[q][j] = -l[q];
+                }
+            }
+        }
+#pragma unroll
+        for (int g = (j & ~3); g < PB; g += 4) {
+            const float4 v4 = *reinterpret_cast<const float4 *>(pr + g);
+            const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int q = 0; q < RPT; ++q)
+                if (live[q]) {
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        if (g + h > j) a[q][g + h] = fmaf(-l[q], v[h], a[q][g + h]);
+                }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = k0 + tid + q * NTH;
+        if (r < n) {
+            perm[pos[q]] = r;
+#pragma unroll
+            for (int j = 0; j < PB; ++j) Lp[j * npad + pos[q]] = a[q][j];
+        }
+    }
+    return true;
+}
+
+// The same with the panel's rows in shared memory (any number of rows).
+template <int PB, int NTH>
+__device__ bool lu_panel_smem(const float *M, int ld, int n, int k0, int kb, float *Lp, int npad, int *perm,
+                              unsigned long long *red, float *red_val)
+{
+    constexpr int NWARP = NTH / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int q = tid; q < (n - k0) * kb; q += NTH) {
+        const int r = k0 + q / kb, j = q - (q / kb) * kb;
+        Lp[j * npad + r] = M[(size_t)r * ld + k0 + j];
+    }
+    for (int r = k0 + tid; r < n; r += NTH) perm[r] = r;
+    __syncthreads();
+    // pivot candidates of the panel's first column
+    {
+        unsigned long long key = 0ull;
+        float kv = 0.f;
+        for (int r = k0 + tid; r < n; r += NTH) {
+            const float v = Lp[r];
+            const unsigned long long kk = piv_key(v, r);
+            if (kk > key) {
+                key = kk;
+                kv = v;
+            }
+        }
+        const unsigned long long wk = warp_max_u64(key);
+        const unsigned ball = __ballot_sync(0xffffffffu, key == wk && wk != 0ull);
+        if (lane == 0) red[warp] = wk;
+        if (ball && lane == __ffs(ball) - 1) red_val[warp] = kv;
+    }
+    __syncthreads();
+    for (int j = 0; j < kb; ++j) {
+        const int c = k0 + j;
+        unsigned long long best = red[0];
+        float pv = red_val[0];
+#pragma unroll
+        for (int q = 1; q < NWARP; ++q)
+            if (red[q] > best) {
+                best = red[q];
+                pv = red_val[q];
+            }
+        const int p = 0x7fffffff - (int)(unsigned)(best & 0xffffffffu);
+        const bool bad = best == 0ull || !(fabsf(pv) > 0.f) || !isfinite(pv);
+        if (!bad && p != c) {
+            if (tid < kb) {
+                const float t = Lp[tid * npad + c];
+                Lp[tid * npad + c] = Lp[tid * npad + p];
+                Lp[tid * npad + p] = t;
+            }
+            if (tid == PB) {
+                const int t = perm[c];
+                perm[c] = perm[p];
+                perm[p] = t;
+            }
+        }
+        __syncthreads();
+        if (bad) return false;
+        // multipliers and the rank-1 update of the panel's remaining
+        // columns; each thread's rows of column j + 1 are final here, so
+        // their pivot candidates are taken on the way
+        const float ipv = 1.0f / pv;
+        unsigned long long key = 0ull;
+        float kv = 0.f;
+        for (int r = c + 1 + tid; r < n; r += NTH) {
+            const float l = Lp[j * npad + r] * ipv;
+            Lp[j * npad + r] = -l;
+            for (int jj = j + 1; jj < kb; ++jj) Lp[jj * npad + r] = fmaf(-l, Lp[jj * npad + c], Lp[jj * npad + r]);
+            if (j + 1 < kb) {
+                const float v = Lp[(j + 1) * npad + r];
                 const unsigned long long kk = piv_key(v, r);
                 if (kk > key) {
                     key = kk;
                     kv = v;
                 }
             }
+        }
+        if (j + 1 < kb) {
             const unsigned long long wk = warp_max_u64(key);
             const unsigned ball = __ballot_sync(0xffffffffu, key == wk && wk != 0ull);
             if (lane == 0) red[warp] = wk;
             if (ball && lane == __ffs(ball) - 1) red_val[warp] = kv;
         }
         __syncthreads();
-        for (int j = 0; j < kb; ++j) {
-            const int c = k0 + j;
-            unsigned long long best = red[0];
-            float pv = red_val[0];
-#pragma unroll
-            for (int q = 1; q < NWARP; ++q)
-                if (red[q] > best) {
-                    best = red[q];
-                    pv = red_val[q];
-                }
-            const int p = 0x7fffffff - (int)(unsigned)(best & 0xffffffffu);
-            const bool bad = best == 0ull || !(fabsf(pv) > 0.f) || !isfinite(pv);
-            if (!bad && p != c) {
-                if (tid < kb) {
-                    const float t = Lp[tid * npad + c];
-                    Lp[tid * npad + c] = Lp[tid * npad + p];
-                    Lp[tid * npad + p] = t;
-                }
-                if (tid == PB) {
-                    const int t = perm[c];
-                    perm[c] = perm[p];
-                    perm[p] = t;
-                }
-            }
+    }
+    return true;
+}
+
+// Solves A X = B in place for the n x w augmented matrix M (row stride ld,
+// A in columns [0, n), right-hand sides in [rhs, w), zero padding between and
+// after), leaving X in rows [row_lo, n) of the right-hand-side columns.
+// RPT: rows of a panel per thread (n <= RPT NTH), 0: panel in shared memory.
+// Returns false if a pivot is zero or not finite.
+template <int PB, int NTH, int RPT>
+__device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int row_lo, float *smem)
+{
+    constexpr int NWARP = NTH / 32;
+    const int tid = threadIdx.x;
+    const int npad = lu_npad(n);
+    float *Lp = smem;
+    float *Us = Lp + (size_t)PB * npad;
+    float *slots = Us + 2 * PB * (UW + 4);
+    int *perm = reinterpret_cast<int *>(slots + (RPT > 0 ? 2 * NWARP * LU_SLOT : 0));
+    int *mv_dst = perm + npad;
+    int *mv_src = mv_dst + PB;
+    int *sh_int = mv_src + PB;                 // [0]: move count
+    unsigned long long *red = reinterpret_cast<unsigned long long *>(sh_int + 8);   // [NWARP]
+    float *red_val = reinterpret_cast<float *>(red + NWARP);                        // [NWARP]
+
+    for (int k0 = 0; k0 < n; k0 += PB) {
+        const int kb = min(PB, n - k0);
+        if (tid == 0) sh_int[0] = 0;
+        if constexpr (RPT > 0) {
+            if (!lu_panel_regs<PB, NTH, RPT>(M, ld, n, k0, kb, Lp, npad, perm, slots)) return false;
             __syncthreads();
-            if (bad) return false;
-            // multipliers and the rank-1 update of the panel's remaining
-            // columns; each thread's rows of column j + 1 are final here, so
-            // their pivot candidates are taken on the way
-            const float ipv = 1.0f / pv;
-            unsigned long long key = 0ull;
-            float kv = 0.f;
-            for (int r = c + 1 + tid; r < n; r += NTH) {
-                const float l = Lp[j * npad + r] * ipv;
-                Lp[j * npad + r] = l;
-                for (int jj = j + 1; jj < kb; ++jj)
-                    Lp[jj * npad + r] = fmaf(-l, Lp[jj * npad + c], Lp[jj * npad + r]);
-                if (j + 1 < kb) {
-                    const float v = Lp[(j + 1) * npad + r];
-                    const unsigned long long kk = piv_key(v, r);
-                    if (kk > key) {
-                        key = kk;
-                        kv = v;
-                    }
-                }
-            }
-            if (j + 1 < kb) {
-                const unsigned long long wk = warp_max_u64(key);
-                const unsigned ball = __ballot_sync(0xffffffffu, key == wk && wk != 0ull);
-                if (lane == 0) red[warp] = wk;
-                if (ball && lane == __ffs(ball) - 1) red_val[warp] = kv;
-            }
-            __syncthreads();
+        } else {
+            if (!lu_panel_smem<PB, NTH>(M, ld, n, k0, kb, Lp, npad, perm, red, red_val)) return false;
         }
-        // rows [k0, k0 + kb) of the panel (U11 and the unit-lower L11) to
-        // global memory; rows moved below the panel by its interchanges
+        // U11 to global memory; rows moved below the panel by its interchanges
         for (int q = tid; q < kb * kb; q += NTH) {
             const int i = q / kb, j = q - (q / kb) * kb;
-            M[(size_t)(k0 + i) * ld + k0 + j] = Lp[j * npad + k0 + i];
+            if (i <= j) M[(size_t)(k0 + i) * ld + k0 + j] = Lp[j * npad + k0 + i];
         }
         for (int r = k0 + kb + tid; r < n; r += NTH)
             if (perm[r] != r) {
@@ -333,14 +502,18 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 for (int i = 0; i < 8; ++i)
                     if (i0 + i < nmv) M[(size_t)mv_dst[i0 + i] * ld + c] = y[i];
             }
+            // x_j -= L_ji x_i, i ascending for every j; four j a shared read
 #pragma unroll
-            for (int j = 1; j < PB; ++j) {
-                if (j < kb) {
-                    float sum = x[j];
+            for (int i = 0; i < PB - 1; ++i) {
+                if (i + 1 < kb) {
 #pragma unroll
-                    for (int i = 0; i < PB; ++i)
-                        if (i < j) sum = fmaf(-Lp[i * npad + k0 + j], x[i], sum);
-                    x[j] = sum;
+                    for (int g = ((i + 1) & ~3); g < PB; g += 4) {
+                        const float4 l = *reinterpret_cast<const float4 *>(Lp + i * npad + k0 + g);
+                        if (g > i) x[g] = fmaf(l.x, x[i], x[g]);
+                        if (g + 1 > i) x[g + 1] = fmaf(l.y, x[i], x[g + 1]);
+                        if (g + 2 > i) x[g + 2] = fmaf(l.z, x[i], x[g + 2]);
+                        if (g + 3 > i) x[g + 3] = fmaf(l.w, x[i], x[g + 3]);
+                    }
                 }
             }
 #pragma unroll
@@ -348,7 +521,7 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 if (j < kb) M[(size_t)(k0 + j) * ld + c] = x[j];
         }
         __syncthreads();
-        if (k0 + kb < n) lu_update_rows<PB>(M, ld, k0, kb, k0 + kb, n, k0 + kb, k0 + kb, w, Lp, npad, Us);
+        if (k0 + kb < n) lu_update_rows<PB, NTH>(M, ld, k0, k0 + kb, n, k0 + kb, k0 + kb, w, Lp, npad, Us);
     }
     // back-substitution of rows [row_lo, n) for the right-hand sides
     const int rs = row_lo & ~3;
@@ -356,9 +529,13 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
     while (t1 > row_lo) {
         const int t0 = max(row_lo, t1 - PB);
         const int tb = t1 - t0;
+        // -U of the block's columns: rows above it into the panel, the block
+        // itself row by row into Us (four columns a read)
         for (int q = tid; q < (t1 - rs) * tb; q += NTH) {
             const int r = rs + q / tb, j = q - (q / tb) * tb;
-            Lp[j * npad + r] = r >= row_lo ? M[(size_t)r * ld + t0 + j] : 0.f;
+            const float v = r >= row_lo ? -M[(size_t)r * ld + t0 + j] : 0.f;
+            if (r < t0) Lp[j * npad + r] = v;
+            else Us[(r - t0) * PB + j] = v;
         }
         __syncthreads();
         for (int c = rhs + tid; c < w; c += NTH) {
@@ -370,9 +547,14 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 if (i < tb) {
                     float sum = x[i];
 #pragma unroll
-                    for (int j = 0; j < PB; ++j)
-                        if (j > i && j < tb) sum = fmaf(-Lp[j * npad + t0 + i], x[j], sum);
-                    x[i] = sum / Lp[i * npad + t0 + i];
+                    for (int g = (i & ~3); g < PB; g += 4) {
+                        const float4 u = *reinterpret_cast<const float4 *>(Us + i * PB + g);
+                        const float v[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (g + j > i && g + j < tb) sum = fmaf(v[j], x[g + j], sum);
+                    }
+                    x[i] = sum / -Us[i * PB + i];
                 }
             }
 #pragma unroll
@@ -380,7 +562,7 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 if (j < tb) M[(size_t)(t0 + j) * ld + c] = x[j];
         }
         __syncthreads();
-        if (t0 > row_lo) lu_update_rows<PB>(M, ld, t0, PB, rs, t0, row_lo, rhs, w, Lp, npad, Us);
+        if (t0 > row_lo) lu_update_rows<PB, NTH>(M, ld, t0, rs, t0, row_lo, rhs, w, Lp, npad, Us);
         t1 = t0;
     }
     return true;
@@ -415,16 +597,40 @@ __device__ __forceinline__ float2 zu(const float2 *Z, int ldz, int i, int j)
     return i <= j ? Z[(size_t)i * ldz + j] : Z[(size_t)j * ldz + i];
 }
 
+// The operands of c -= a b with packed FMAs: b1 = (b.y, -b.x), b2 = -b; then
+// c = fma2((a.x, a.x), b2, fma2((a.y, a.y), b1, c)) rounds as cfma_neg does.
+__device__ __forceinline__ float4 zpair(float2 b) { return make_float4(b.y, -b.x, -b.x, -b.y); }
+
+// How a multiplicand is kept in shared memory: as its pair, or (LEAN) itself.
+template <bool LEAN> struct ZOp {
+    using type = float4;
+    static __device__ __forceinline__ float4 make(float2 b) { return zpair(b); }
+};
+template <> struct ZOp<true> {
+    using type = float2;
+    static __device__ __forceinline__ float2 make(float2 b) { return b; }
+};
+__device__ __forceinline__ ulonglong2 zget(const float4 *p) { return *reinterpret_cast<const ulonglong2 *>(p); }
+__device__ __forceinline__ ulonglong2 zget(const float2 *p)
+{
+    const float4 q = zpair(*p);
+    return make_ulonglong2(pack2(q.x, q.y), pack2(q.z, q.w));
+}
+
 // Z (m x m complex symmetric, row stride ldz, zero padding to ldz) <- -Z^{-1}
 // in its upper triangle (the lower triangle is left stale).
-template <int PB>
+template <int PB, int NTH, bool LEAN>
 __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
 {
+    using Op = typename ZOp<LEAN>::type;
+    constexpr int TR = NTH / 4;                   // rows per tile
+    constexpr int SPT = PB * UWC / NTH;           // strip elements per thread
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int npz = z_npad(m);
     float2 *Lp = smem;
-    float2 *Us = Lp + (size_t)PB * npz;
-    float2 *Bs = Us + PB * (UWC + 2);
+    Op *Us = reinterpret_cast<Op *>(Lp + (size_t)PB * npz);   // two strips (LEAN: one)
+    Op *Bp = Us + (LEAN ? 1 : 2) * PB * (UWC + 2);
+    float2 *Bs = reinterpret_cast<float2 *>(Bp + (LEAN ? 0 : PB * PB));
     for (int k0 = 0; k0 < m; k0 += PB) {
         const int kb = min(PB, m - k0);
         if (tid < PB * PB) {
@@ -437,11 +643,11 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
             const float2 d = Bs[p * (PB + 1) + p];
             const bool bad = !(fabsf(d.x) + fabsf(d.y) > 0.f) || !isfinite(d.x) || !isfinite(d.y);
             if (bad) return false;   // the same decision in every thread
-            const float2 dinv = crcp_safe(d);
             float2 v = make_float2(0.f, 0.f);
             const int i = tid / PB, j = tid - (tid / PB) * PB;
             const bool own = tid < PB * PB && i < kb && j < kb;
             if (own) {
+                const float2 dinv = crcp_safe(d);
                 if (i == p && j == p) {
                     v = make_float2(-dinv.x, -dinv.y);
                 } else if (i == p) {
@@ -456,100 +662,147 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
             if (own) Bs[i * (PB + 1) + j] = v;
             __syncthreads();
         }
-        // panel P_i = Z[i, K] B^{-1} = -Z[i, K] Bs for rows i outside K
-        for (int i = tid; i < m; i += NTH) {
-            float2 P[PB];
+        if constexpr (!LEAN) {
+            if (tid < PB * PB) Bp[tid] = zpair(Bs[(tid / PB) * (PB + 1) + (tid - (tid / PB) * PB)]);
+            __syncthreads();
+        }
+        // panel P_i = Z[i, K] B^{-1} = -Z[i, K] Bs for rows i outside K; a
+        // thread takes half a row's columns
+        for (int t = tid; t < 2 * m; t += NTH) {
+            const int i = t < m ? t : t - m, kh = t < m ? 0 : PB / 2;
+            unsigned long long P[PB / 2];
 #pragma unroll
-            for (int k = 0; k < PB; ++k) P[k] = make_float2(0.f, 0.f);
+            for (int k = 0; k < PB / 2; ++k) P[k] = 0ull;
             if (i < k0 || i >= k0 + kb) {
+                float2 zq[PB];
+#pragma unroll
+                for (int q = 0; q < PB; ++q) zq[q] = q < kb ? zu(Z, ldz, i, k0 + q) : make_float2(0.f, 0.f);
 #pragma unroll
                 for (int q = 0; q < PB; ++q) {
                     if (q < kb) {
-                        const float2 zq = zu(Z, ldz, i, k0 + q);
+                        const unsigned long long ax = pack2(zq[q].x, zq[q].x), ay = pack2(zq[q].y, zq[q].y);
 #pragma unroll
-                        for (int k = 0; k < PB; ++k) P[k] = cfma_neg(zq, Bs[q * (PB + 1) + k], P[k]);
+                        for (int k = 0; k < PB / 2; ++k) {
+                            ulonglong2 b;
+                            if constexpr (LEAN) b = zget(Bs + q * (PB + 1) + kh + k);
+                            else b = zget(Bp + q * PB + kh + k);
+                            P[k] = fma2(ax, b.y, fma2(ay, b.x, P[k]));
+                        }
                     }
                 }
             }
 #pragma unroll
-            for (int k = 0; k < PB; ++k) Lp[k * npz + i] = (k < kb) ? P[k] : make_float2(0.f, 0.f);
+            for (int k = 0; k < PB / 2; ++k)
+                Lp[(kh + k) * npz + i] = (kh + k < kb) ? unpack2(P[k]) : make_float2(0.f, 0.f);
         }
-        __syncthreads();
-        // Z_ij -= P_i Z_Kj for i, j outside K, i <= j (tiles of 128 x 64
-        // wholly below the diagonal are skipped), 64 columns at a time
-        for (int c0 = 0; c0 < m; c0 += UWC) {
-            for (int q = tid; q < PB * UWC; q += NTH) {
-                const int k = q / UWC, jj = q - (q / UWC) * UWC;
-                const int c = c0 + jj;
+        // Z_ij -= P_i Z_Kj for i, j outside K, i <= j (tiles of TR x 64
+        // wholly below the diagonal are skipped), 64 columns at a time; the
+        // next strip's Z_Kj and the next tile's Z_ij are on their way meanwhile
+        const int nstrip = (m + UWC - 1) / UWC;
+        float2 st[SPT];
+        auto fetch = [&](int s) {   // strips left of K lie in columns of Z: k fastest there
+            const bool left = s * UWC < k0;
+#pragma unroll
+            for (int u = 0; u < SPT; ++u) {
+                const int q = tid + u * NTH;
+                const int k = left ? q % PB : q / UWC, c = s * UWC + (left ? q / PB : q % UWC);
                 const bool in = k < kb && c < m && (c < k0 || c >= k0 + kb);
-                Us[k * (UWC + 2) + jj] = in ? zu(Z, ldz, k0 + k, c) : make_float2(0.f, 0.f);
+                st[u] = in ? zu(Z, ldz, k0 + k, c) : make_float2(0.f, 0.f);
             }
-            __syncthreads();
-            const int cb[2] = {c0 + 2 * tx, c0 + 32 + 2 * tx};
+        };
+        auto put = [&](int s) {
+            const bool left = s * UWC < k0;
+            Op *buf = Us + (LEAN ? 0 : (s & 1)) * PB * (UWC + 2);
+#pragma unroll
+            for (int u = 0; u < SPT; ++u) {
+                const int q = tid + u * NTH;
+                const int k = left ? q % PB : q / UWC, jj = left ? q / PB : q % UWC;
+                // column 32 h + 2 x + e of the strip at 16 (2 h + e) + x: a
+                // thread's four columns are four conflict-free reads
+                buf[k * (UWC + 2) + 16 * (2 * (jj >> 5) + (jj & 1)) + ((jj & 31) >> 1)] = ZOp<LEAN>::make(st[u]);
+            }
+        };
+        auto zload = [&](int rb, int c0, unsigned long long (&v)[4][4]) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = rb + i;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int c = c0 + 32 * h + 2 * tx;
+                    ulonglong2 q = make_ulonglong2(0ull, 0ull);
+                    if (r < m && c < ldz) q = *reinterpret_cast<const ulonglong2 *>(Z + (size_t)r * ldz + c);
+                    v[i][2 * h] = q.x;
+                    v[i][2 * h + 1] = q.y;
+                }
+            }
+        };
+        unsigned long long acc[4][4], nxt[4][4];
+        fetch(0);
+        if (!LEAN) put(0);
+        const int rb0 = ty * 4;
+        zload(rb0, 0, acc);
+        for (int s = 0; s < nstrip; ++s) {
+            const int c0 = s * UWC;
+            const Op *cur = Us + (LEAN ? 0 : (s & 1)) * PB * (UWC + 2);
+            if (LEAN) {
+                __syncthreads();
+                put(s);
+            }
+            __syncthreads();   // strip s (and, the first time, the panel) is complete
+            if (s + 1 < nstrip) fetch(s + 1);
             const int r_end = min(m, c0 + UWC);   // row tiles starting past this are below the diagonal
-            auto zload = [&](int rb, float2 (&v)[4][4]) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = rb + i;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (r < m && cb[h] < ldz) q = *reinterpret_cast<const float4 *>(Z + (size_t)r * ldz + cb[h]);
-                        v[i][2 * h] = make_float2(q.x, q.y);
-                        v[i][2 * h + 1] = make_float2(q.z, q.w);
-                    }
-                }
-            };
-            float2 acc[4][4], nxt[4][4];
-            int rb = ty * 4;
-            if (rb < m) zload(rb, acc);
-            for (int r0 = 0; r0 < r_end; r0 += 128, rb += 128) {
-                if (rb >= m) break;
-                if (r0 + 128 < r_end && rb + 128 < m) zload(rb + 128, nxt);
+            int rb = rb0;
+            for (int r0 = 0; r0 < r_end; r0 += TR, rb += TR) {
+                const bool last = r0 + TR >= r_end;
+                if (!last) zload(rb + TR, c0, nxt);
+                else if (s + 1 < nstrip) zload(rb0, c0 + UWC, nxt);
+                if (rb < m) {
 #pragma unroll 4
-                for (int k = 0; k < PB; ++k) {
-                    float2 a[4], b[4];
-                    const float4 a0 = *reinterpret_cast<const float4 *>(Lp + k * npz + rb);
-                    const float4 a1 = *reinterpret_cast<const float4 *>(Lp + k * npz + rb + 2);
-                    a[0] = make_float2(a0.x, a0.y);
-                    a[1] = make_float2(a0.z, a0.w);
-                    a[2] = make_float2(a1.x, a1.y);
-                    a[3] = make_float2(a1.z, a1.w);
-                    const float4 b0 = *reinterpret_cast<const float4 *>(Us + k * (UWC + 2) + 2 * tx);
-                    const float4 b1 = *reinterpret_cast<const float4 *>(Us + k * (UWC + 2) + 32 + 2 * tx);
-                    b[0] = make_float2(b0.x, b0.y);
-                    b[1] = make_float2(b0.z, b0.w);
-                    b[2] = make_float2(b1.x, b1.y);
-                    b[3] = make_float2(b1.z, b1.w);
+                    for (int k = 0; k < PB; ++k) {
+                        const float4 a0 = *reinterpret_cast<const float4 *>(Lp + k * npz + rb);
+                        const float4 a1 = *reinterpret_cast<const float4 *>(Lp + k * npz + rb + 2);
+                        const Op *b = cur + k * (UWC + 2) + tx;
+                        const ulonglong2 b0 = zget(b), b1 = zget(b + 16), b2 = zget(b + 32), b3 = zget(b + 48);
+                        const float ax[4] = {a0.x, a0.z, a1.x, a1.z}, ay[4] = {a0.y, a0.w, a1.y, a1.w};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                        for (int i = 0; i < 4; ++i) {
+                            const unsigned long long y = pack2(ay[i], ay[i]), x = pack2(ax[i], ax[i]);
+                            acc[i][0] = fma2(y, b0.x, acc[i][0]);
+                            acc[i][1] = fma2(y, b1.x, acc[i][1]);
+                            acc[i][2] = fma2(y, b2.x, acc[i][2]);
+                            acc[i][3] = fma2(y, b3.x, acc[i][3]);
+                            acc[i][0] = fma2(x, b0.y, acc[i][0]);
+                            acc[i][1] = fma2(x, b1.y, acc[i][1]);
+                            acc[i][2] = fma2(x, b2.y, acc[i][2]);
+                            acc[i][3] = fma2(x, b3.y, acc[i][3]);
+                        }
+                    }
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = cfma_neg(a[i], b[j], acc[i][j]);
-                }
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = rb + i;
+                        if (r >= m) continue;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = rb + i;
-                    if (r >= m) continue;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if (cb[h] < ldz)
-                            *reinterpret_cast<float4 *>(Z + (size_t)r * ldz + cb[h]) =
-                                make_float4(acc[i][2 * h].x, acc[i][2 * h].y, acc[i][2 * h + 1].x,
-                                            acc[i][2 * h + 1].y);
+                        for (int h = 0; h < 2; ++h) {
+                            const int c = c0 + 32 * h + 2 * tx;
+                            if (c < ldz)
+                                *reinterpret_cast<ulonglong2 *>(Z + (size_t)r * ldz + c) =
+                                    make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
+                        }
+                    }
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) acc[i][j] = nxt[i][j];
             }
-            __syncthreads();
+            if (!LEAN && s + 1 < nstrip) put(s + 1);
         }
+        __syncthreads();
         // upper-triangle positions of Z[i, K] = P_i and Z[K, i] = P_i^T, and
         // Z[K, K] = -B^{-1}
-        for (int i = tid; i < k0; i += NTH) {
-#pragma unroll
-            for (int k = 0; k < PB; ++k)
-                if (k < kb) Z[(size_t)i * ldz + k0 + k] = Lp[k * npz + i];
+        for (int q = tid; q < k0 * PB; q += NTH) {
+            const int i = q / PB, k = q - (q / PB) * PB;
+            if (k < kb) Z[(size_t)i * ldz + k0 + k] = Lp[k * npz + i];
         }
         for (int q = tid; q < kb * (m - k0 - kb); q += NTH) {
             const int k = q / (m - k0 - kb), i = k0 + kb + (q - (q / (m - k0 - kb)) * (m - k0 - kb));

@@ -17,7 +17,7 @@
 //
 // FP64 by default. With the FP32 matching option (rm_opts.solve_precision =
 // RM_FP32) the matching system is assembled and solved in FP32 and the T step
-// inverts 1 - iK in FP32 complex arithmetic (dense_global_f32.cuh: one CTA per
+// inverts 1 - iK in FP32 complex arithmetic (dense_global_f32.cuh: a CTA per
 // energy, blocked LU with partial pivoting; blocked sweep of the complex
 // symmetric 1 - iK), while the MQDT elimination, K and Omega stay FP64:
 //
@@ -672,8 +672,8 @@ __global__ void assemble_f32_kernel(PwDev pw, int nE, const ChanFn *__restrict__
     }
 }
 
-template <int PB>
-__global__ void __launch_bounds__(f32d::NTH, 1) lu32_kernel(int n, const EnergyDims *__restrict__ dims, double *ws,
+template <int PB, int NT, int RPT>
+__global__ void __launch_bounds__(NT, 512 / NT) lu32_kernel(int n, const EnergyDims *__restrict__ dims, double *ws,
                                                             int *status, const int *__restrict__ order)
 {
     extern __shared__ float4 fsm4[];
@@ -682,8 +682,8 @@ __global__ void __launch_bounds__(f32d::NTH, 1) lu32_kernel(int n, const EnergyD
     if (d.np < 0) return;
     float *M = reinterpret_cast<float *>(slot_of(ws, n, e).aug);
     const int rhs = f32d::rhs0(n);
-    if (!f32d::lu32_factor_solve<PB>(M, f32d::aug_ld(n, d.np), n, rhs + d.np, rhs, d.ncl,
-                                     reinterpret_cast<float *>(fsm4)))
+    if (!f32d::lu32_factor_solve<PB, NT, RPT>(M, f32d::aug_ld(n, d.np), n, rhs + d.np, rhs, d.ncl,
+                                              reinterpret_cast<float *>(fsm4)))
         if (threadIdx.x == 0) atomicCAS(status + e, RM_OK, RM_ESINGULAR);
 }
 
@@ -725,8 +725,8 @@ __global__ void zbuild_kernel(int n, int nE, const EnergyDims *dims, double *ws)
     }
 }
 
-template <int PB>
-__global__ void __launch_bounds__(f32d::NTH, 1) zsweep_kernel(int n, const EnergyDims *__restrict__ dims, double *ws,
+template <int PB, int NT, bool LEAN>
+__global__ void __launch_bounds__(NT, 512 / NT) zsweep_kernel(int n, const EnergyDims *__restrict__ dims, double *ws,
                                                               int *status, const int *__restrict__ order)
 {
     extern __shared__ float4 fsm4[];
@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(f32d::NTH, 1) zsweep_kernel(int n, const Energ
     const EnergyDims d = dims[e];
     if (d.np < 0) return;
     float2 *Z = reinterpret_cast<float2 *>(slot_of(ws, n, e).aug);
-    if (!f32d::zsweep_invert<PB>(Z, f32d::z_ld(d.no), d.no, reinterpret_cast<float2 *>(fsm4)))
+    if (!f32d::zsweep_invert<PB, NT, LEAN>(Z, f32d::z_ld(d.no), d.no, reinterpret_cast<float2 *>(fsm4)))
         if (threadIdx.x == 0) atomicCAS(status + e, RM_OK, RM_ESINGULAR);
 }
 
@@ -771,23 +771,76 @@ int max_dyn_smem()
     return v;
 }
 
+template <class K> cudaError_t set_smem(K kern, size_t bytes)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // Panel widths that fit shared memory for n channels (0: none fits).
 int lu_pb(int n)
 {
-    if (f32d::lu_smem<32>(n) <= (size_t)max_dyn_smem()) return 32;
-    if (f32d::lu_smem<16>(n) <= (size_t)max_dyn_smem()) return 16;
+    if (f32d::lu_smem<32, 512, 0>(n) <= (size_t)max_dyn_smem()) return 32;
+    if (f32d::lu_smem<16, 512, 0>(n) <= (size_t)max_dyn_smem()) return 16;
     return 0;
 }
 int z_pb(int m)
 {
-    if (f32d::z_smem<16>(m) <= (size_t)max_dyn_smem()) return 16;
-    if (f32d::z_smem<8>(m) <= (size_t)max_dyn_smem()) return 8;
+    if (f32d::z_smem<16, true>(m) <= (size_t)max_dyn_smem()) return 16;
+    if (f32d::z_smem<8, true>(m) <= (size_t)max_dyn_smem()) return 8;
     return 0;
 }
 
-template <class K> cudaError_t set_smem(K kern, size_t bytes)
+template <int PB, int NT, int RPT>
+cudaError_t launch_lu32(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order, cudaStream_t st)
 {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const size_t sm = f32d::lu_smem<PB, NT, RPT>(n);
+    const cudaError_t err = set_smem(lu32_kernel<PB, NT, RPT>, sm);
+    if (err != cudaSuccess) return err;
+    lu32_kernel<PB, NT, RPT><<<nE, NT, sm, st>>>(n, dims, ws, status, order);
+    return cudaGetLastError();
+}
+
+// A panel's rows in the registers of 256 threads (two CTAs per SM) up to 256
+// channels, of 512 up to 512 (203 unknowns: 1.11 ms per 912 systems; two rows
+// a thread on 256 threads are slower at 431, 3.89 against 3.44 ms per 456),
+// two rows a thread up to 1024; in shared memory above.
+cudaError_t launch_lu32_any(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
+                            cudaStream_t st)
+{
+    if (n <= 256) return launch_lu32<32, 256, 1>(n, nE, dims, ws, status, order, st);
+    if (n <= 512) return launch_lu32<32, 512, 1>(n, nE, dims, ws, status, order, st);
+    if (n <= 1024) return launch_lu32<32, 512, 2>(n, nE, dims, ws, status, order, st);
+    if (lu_pb(n) == 32) return launch_lu32<32, 512, 0>(n, nE, dims, ws, status, order, st);
+    return launch_lu32<16, 512, 0>(n, nE, dims, ws, status, order, st);
+}
+
+template <int PB, int NT, bool LEAN>
+cudaError_t launch_zsweep(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
+                          cudaStream_t st)
+{
+    const size_t sm = f32d::z_smem<PB, LEAN>(n);
+    const cudaError_t err = set_smem(zsweep_kernel<PB, NT, LEAN>, sm);
+    if (err != cudaSuccess) return err;
+    zsweep_kernel<PB, NT, LEAN><<<nE, NT, sm, st>>>(n, dims, ws, status, order);
+    return cudaGetLastError();
+}
+
+// Two CTAs of 256 threads per SM while their shared memory fits (up to 512
+// channels: 300 open ones 2.30 against 2.76 ms per 456 systems on 512
+// threads; 500 open 6.80 against 6.57 ms per 304). The pivots per block (16,
+// above 1733 channels 8) decide the rounding and do not depend on this.
+cudaError_t launch_zsweep_any(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
+                              cudaStream_t st)
+{
+    if (n <= 512) return launch_zsweep<16, 256, false>(n, nE, dims, ws, status, order, st);
+    if (z_pb(n) == 16) {
+        if (f32d::z_smem<16, false>(n) <= (size_t)max_dyn_smem())
+            return launch_zsweep<16, 512, false>(n, nE, dims, ws, status, order, st);
+        return launch_zsweep<16, 512, true>(n, nE, dims, ws, status, order, st);
+    }
+    if (f32d::z_smem<8, false>(n) <= (size_t)max_dyn_smem())
+        return launch_zsweep<8, 512, false>(n, nE, dims, ws, status, order, st);
+    return launch_zsweep<8, 512, true>(n, nE, dims, ws, status, order, st);
 }
 
 }  // namespace
@@ -848,16 +901,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
         LAUNCH_OK();
         assemble_f32_kernel<<<dim3(xb, nE), NTH, 0, st>>>(pw, nE, cf, R, dims, col_chan, ws);
         LAUNCH_OK();
-        const int pb = lu_pb(n);
-        if (pb == 32) {
-            const size_t sm = f32d::lu_smem<32>(n);
-            if ((err = set_smem(lu32_kernel<32>, sm)) != cudaSuccess) return err;
-            lu32_kernel<32><<<nE, f32d::NTH, sm, st>>>(n, dims, ws, status, order);
-        } else {
-            const size_t sm = f32d::lu_smem<16>(n);
-            if ((err = set_smem(lu32_kernel<16>, sm)) != cudaSuccess) return err;
-            lu32_kernel<16><<<nE, f32d::NTH, sm, st>>>(n, dims, ws, status, order);
-        }
+        if ((err = launch_lu32_any(n, nE, dims, ws, status, order, st)) != cudaSuccess) return err;
         LAUNCH_OK();
         prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
         LAUNCH_OK();
@@ -892,16 +936,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
     if (omega && f32) {
         zbuild_kernel<<<dim3(xb2, nE), NTH, 0, st>>>(n, nE, dims, ws);
         LAUNCH_OK();
-        const int pb = z_pb(n);
-        if (pb == 16) {
-            const size_t sm = f32d::z_smem<16>(n);
-            if ((err = set_smem(zsweep_kernel<16>, sm)) != cudaSuccess) return err;
-            zsweep_kernel<16><<<nE, f32d::NTH, sm, st>>>(n, dims, ws, status, order);
-        } else {
-            const size_t sm = f32d::z_smem<8>(n);
-            if ((err = set_smem(zsweep_kernel<8>, sm)) != cudaSuccess) return err;
-            zsweep_kernel<8><<<nE, f32d::NTH, sm, st>>>(n, dims, ws, status, order);
-        }
+        if ((err = launch_zsweep_any(n, nE, dims, ws, status, order, st)) != cudaSuccess) return err;
         LAUNCH_OK();
         prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
         LAUNCH_OK();
