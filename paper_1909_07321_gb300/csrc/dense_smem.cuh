@@ -105,7 +105,7 @@ __device__ void block_backsub(T *M, int ld, int rows, int rhs0, int n_rhs, int r
 // k, with d = a_kk and v_i = a_ik / d: a_ij -= v_i v_j d (i, j != k),
 // a_ik = v_i, a_kk = -1/d; after all m steps the upper triangle holds
 // -A^{-1}, which is then negated and mirrored into the full matrix.
-// v is shared scratch of m doubles. Sets sh->bad if a pivot is not positive.
+// v is shared scratch of m <= NT doubles. Sets sh->bad if a pivot is not positive.
 __device__ void spd_sweep_inverse(double *A, int ld, int m, double *v, ElimShared *sh)
 {
     const int tid = threadIdx.x;
@@ -117,10 +117,15 @@ __device__ void spd_sweep_inverse(double *A, int ld, int m, double *v, ElimShare
             if (tid == 0) sh->bad = 1;
             return;
         }
-        const double dinv = 1.0 / d;
-        for (int i = tid; i < m; i += NT)
-            v[i] = (i == k) ? 0.0 : ((i < k) ? A[i * ld + k] : A[k * ld + i]) * dinv;
+        // the division takes a warp about 12 FP64 instructions of 64 clocks of
+        // its quarter of the FP64 unit each: only the warps holding v take it
+        if (tid < ((m + 31) & ~31)) {
+            const double dinv = 1.0 / d;
+            if (tid < m) v[tid] = (tid == k) ? 0.0 : ((tid < k) ? A[tid * ld + k] : A[k * ld + tid]) * dinv;
+            if (tid == 0) sh->pivinv = dinv;
+        }
         __syncthreads();
+        const double dinv = sh->pivinv;
         for (int q = tid; q < ngroups * G; q += NT) {
             const int g = q / G, t = q - (q / G) * G;
             for (int h = 0; h < 2; ++h) {
@@ -185,18 +190,17 @@ __device__ __forceinline__ void tri_pair(int q, int m, int &p, int &r)
 //   K = K_oo - K_oc (K_cc + diag(tq))^{-1} K_co
 // from K_u (np x np, row stride lu) with the eliminated channels at P
 // positions qpos[0..nq) and the open ones at opos[0..no); tq[i] is the
-// diagonal term of eliminated channel i (tan pi nu). scratch holds
-// nq (nq + no + 1) + no (no + 1) doubles. K is written symmetrised to Ks
-// (row stride no + 1; Ks may be K_u's storage, which is not read after the
-// product is formed) and, unsymmetrised, to K_row (row stride ldo) when not
-// null. Returns false (sh->bad set) if K_cc + diag(tq) is singular.
+// diagonal term of eliminated channel i (tan pi nu). C (nq x (nq + no), row
+// stride ld2) and Kd (no x no, row stride lkd) are scratch. K is written
+// symmetrised to Ks (row stride lks; Ks may be K_u's storage, which is not read
+// after the product is formed) and, unsymmetrised, to K_row (row stride ldo)
+// when not null. Returns false (sh->bad set) if K_cc + diag(tq) is singular.
 __device__ bool mqdt_eliminate(const double *Ku, int lu, int no, int nq, const int *qpos, const int *opos,
-                               const double *tq, double *scratch, double *Ks, double *K_row, int ldo,
-                               ElimShared *sh)
+                               const double *tq, double *C, int ld2, double *Kd, int lkd, double *Ks, int lks,
+                               double *K_row, int ldo, ElimShared *sh)
 {
     const int tid = threadIdx.x;
-    const int w2 = nq + no, ld2 = w2 + 1, lk = no + 1;
-    double *C = scratch;
+    const int w2 = nq + no;
     for (int q = tid; q < nq * w2; q += NT) {
         const int i = q / w2, j = q - (q / w2) * w2;
         double v;
@@ -212,18 +216,17 @@ __device__ bool mqdt_eliminate(const double *Ku, int lu, int no, int nq, const i
     block_eliminate<double>(C, ld2, nq, w2, sh);
     if (sh->bad) return false;
     block_backsub<double>(C, ld2, nq, nq, no, 0);   // Y = (K_cc + tq)^{-1} K_co
-    double *Kd = scratch + (size_t)nq * ld2;
     for (int q = tid; q < no * no; q += NT) {
         const int s2 = q / no, t = q - (q / no) * no;
         double v = Ku[opos[s2] * lu + opos[t]];
         for (int i = 0; i < nq; ++i) v = fma(-Ku[opos[s2] * lu + qpos[i]], C[i * ld2 + nq + t], v);
-        Kd[s2 * lk + t] = v;
+        Kd[s2 * lkd + t] = v;
     }
     __syncthreads();
     for (int q = tid; q < no * no; q += NT) {
         const int p = q / no, r = q - (q / no) * no;
-        const double kpr = Kd[p * lk + r];
-        Ks[p * lk + r] = 0.5 * (kpr + Kd[r * lk + p]);
+        const double kpr = Kd[p * lkd + r];
+        Ks[p * lks + r] = 0.5 * (kpr + Kd[r * lkd + p]);
         if (K_row) K_row[(size_t)p * ldo + r] = kpr;
     }
     __syncthreads();

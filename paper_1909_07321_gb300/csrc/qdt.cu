@@ -222,10 +222,19 @@ __device__ __forceinline__ double2 crcp(double2 a)
 
 // Complex Gaussian elimination with partial pivoting of the first `rows`
 // columns of the rows x w matrix M (row stride ld). Sets sh->bad on a zero
-// or non-finite pivot.
-__device__ void cblock_eliminate(double2 *M, int ld, int rows, int w, ElimShared *sh, double2 *pinv_s)
+// or non-finite pivot. orig (or nullptr, shared, rows ints): the right-hand
+// sides are the unit matrix (w = 2 rows); the pivot row of step c is nonzero
+// only in the c + 1 right-hand columns of the rows that have been pivots
+// (orig[0..c]), and the others, which subtract zeros, are left out.
+template <int NTH>
+__device__ void cblock_eliminate(double2 *M, int ld, int rows, int w, ElimShared *sh, double2 *pinv_s,
+                                 int *orig = nullptr)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (orig) {
+        for (int r = tid; r < rows; r += NTH) orig[r] = r;
+        __syncthreads();
+    }
     for (int c = 0; c < rows; ++c) {
         if (warp == 0) {
             double best = -1.0;
@@ -251,42 +260,77 @@ __device__ void cblock_eliminate(double2 *M, int ld, int rows, int w, ElimShared
         if (sh->bad) return;
         const int p = sh->piv;
         if (p != c) {
-            for (int q = c + tid; q < w; q += NT) {
+            for (int q = c + tid; q < w; q += NTH) {
                 const double2 t = M[c * ld + q];
                 M[c * ld + q] = M[p * ld + q];
                 M[p * ld + q] = t;
             }
+            if (orig && tid == NTH - 1) {
+                const int t = orig[c];
+                orig[c] = orig[p];
+                orig[p] = t;
+            }
             __syncthreads();
         }
-        constexpr int G = 4;
+        constexpr int G = NTH / 64;
         const double2 pinv = *pinv_s;
         const int nr = rows - c - 1;
+        const int wl = orig ? rows : w;
         const double2 *prow = M + c * ld;
-        for (int q = tid; q < nr * G; q += NT) {
+        for (int q = tid; q < nr * G; q += NTH) {
             const int r = c + 1 + q / G, j = q - (q / G) * G;
             double2 *row = M + r * ld;
             const double2 f = cmul(row[c], pinv);
-            for (int cc = c + 1 + j; cc < w; cc += G) row[cc] = cfms(row[cc], f, prow[cc]);
+            for (int cc = c + 1 + j; cc < wl; cc += G) row[cc] = cfms(row[cc], f, prow[cc]);
+            if (orig)
+                for (int k = j; k <= c; k += G) {
+                    const int cc = rows + orig[k];
+                    row[cc] = cfms(row[cc], f, prow[cc]);
+                }
         }
         __syncthreads();
     }
 }
 
+// A pair of lanes per right-hand side, one for the real and one for the
+// imaginary part: each row's sum is one serial chain, half as long this way.
+template <int NTH>
 __device__ void cblock_backsub(double2 *M, int ld, int rows, int rhs0, int n_rhs)
 {
-    for (int qq = threadIdx.x; qq < n_rhs; qq += NT) {
-        const int cq = rhs0 + qq;
+    for (int q0 = 0; q0 < n_rhs; q0 += NTH / 2) {
+        const int qq = q0 + (threadIdx.x >> 1);
+        const bool im = threadIdx.x & 1;
+        // whole warps take part in the exchanges
+        if (q0 + ((threadIdx.x & ~31) >> 1) >= n_rhs) break;
+        const bool on = qq < n_rhs;
+        const int cq = rhs0 + (on ? qq : 0);
         for (int t = rows - 1; t >= 0; --t) {
-            double2 s = M[t * ld + cq];
-            for (int u = t + 1; u < rows; ++u) s = cfms(s, M[t * ld + u], M[u * ld + cq]);
-            M[t * ld + cq] = cmul(s, crcp(M[t * ld + t]));
+            const double2 s0 = M[t * ld + cq];
+            double s = im ? s0.y : s0.x;
+            for (int u = t + 1; u < rows; ++u) {
+                const double2 b = M[t * ld + u], c = M[u * ld + cq];
+                // cfms: x - (b.x c.x - b.y c.y), y - (b.x c.y + b.y c.x)
+                const double lo = im ? b.y * c.x : -b.y * c.y;
+                s = s - fma(b.x, im ? c.y : c.x, lo);
+            }
+            const double o = __shfl_xor_sync(0xffffffffu, s, 1);
+            const double2 v = cmul(im ? make_double2(o, s) : make_double2(s, o), crcp(M[t * ld + t]));
+            __syncwarp();
+            if (on) {
+                if (im) M[t * ld + cq].y = v.y;
+                else M[t * ld + cq].x = v.x;
+            }
+            __syncwarp();
         }
     }
     __syncthreads();
 }
 
 // Node K_u -> S_u = 2 (1 - i K_u)^{-1} - 1: one CTA per node, [A | I] eliminated.
-__global__ void __launch_bounds__(NT) qdt_s_from_k_kernel(int n, const double *__restrict__ Ku,
+// One CTA per SM (the 64 x 128 complex system takes 132 KB), so 512 threads.
+// 389 nodes of 64 channels: 1.32 ms, were 1.70.
+constexpr int NTS = 512;
+__global__ void __launch_bounds__(NTS) qdt_s_from_k_kernel(int n, const double *__restrict__ Ku,
                                                          const int *__restrict__ np_node,
                                                          int *__restrict__ status,
                                                          double2 *__restrict__ Su)
@@ -294,13 +338,14 @@ __global__ void __launch_bounds__(NT) qdt_s_from_k_kernel(int n, const double *_
     extern __shared__ double2 smc[];
     __shared__ ElimShared esh;
     __shared__ double2 pinv_s;
+    __shared__ int orig[SOLVE_SMALL_MAXN];
     const int k = blockIdx.x, tid = threadIdx.x;
     if (status[k] != RM_OK) return;
     const int m = np_node[k];
     const int w = 2 * m, ld = w + 1;
     const double *K = Ku + (size_t)k * n * n;
     if (tid == 0) esh.bad = 0;
-    for (int q = tid; q < m * w; q += NT) {
+    for (int q = tid; q < m * w; q += NTS) {
         const int r = q / w, c = q - (q / w) * w;
         double2 v;
         if (c < m) v = make_double2(r == c ? 1.0 : 0.0, -K[(size_t)r * n + c]);
@@ -308,14 +353,14 @@ __global__ void __launch_bounds__(NT) qdt_s_from_k_kernel(int n, const double *_
         smc[r * ld + c] = v;
     }
     __syncthreads();
-    cblock_eliminate(smc, ld, m, w, &esh, &pinv_s);
+    cblock_eliminate<NTS>(smc, ld, m, w, &esh, &pinv_s, orig);
     if (esh.bad) {   // an unusable node: left out through its status
         if (tid == 0) status[k] = RM_ESINGULAR;
         return;
     }
-    cblock_backsub(smc, ld, m, m, m);
+    cblock_backsub<NTS>(smc, ld, m, m, m);
     double2 *S = Su + (size_t)k * n * n;
-    for (int q = tid; q < m * m; q += NT) {
+    for (int q = tid; q < m * m; q += NTS) {
         const int r = q / m, c = q - (q / m) * m;
         const double2 v = smc[r * ld + m + c];
         S[(size_t)r * n + c] = make_double2(2.0 * v.x - (r == c ? 1.0 : 0.0), 2.0 * v.y);
@@ -345,32 +390,47 @@ __global__ void __launch_bounds__(NT) qdt_fine_kernel(PwDev pw, const double *__
     const int n = pw.n;
     const double x = E[e];
     const QdtFine f = fine[e];
+    // classes of the channels (a thread each: one thread's square roots and
+    // sines of all closed channels took 40 us an energy), then their positions
+    __shared__ signed char cls[SOLVE_SMALL_MAXN];
+    __shared__ double tanv[SOLVE_SMALL_MAXN];
+    __shared__ double2 dqv[SOLVE_SMALL_MAXN];
+    int flag = f.flag;
+    if (flag == QDT_FLAG_OK && (node_status[f.a] != RM_OK || node_status[f.b] != RM_OK)) flag = QDT_FLAG_NONODE;
+    bool open = false;
+    if (tid < n) {
+        const double eps = x - pw.e_thr[tid];
+        open = eps > 0.0;
+        signed char c = QDT_DECAY;
+        if (open) {
+            c = QDT_OPEN;
+        } else if (pw.z > 0.0 && flag == QDT_FLAG_OK) {
+            const double kap = sqrt(-eps);
+            const double nu = pw.z / kap;
+            if (nu >= fmax(pw.l[tid] + o.nu_margin, o.fnumin) && kap * pw.a <= o.kappa_a_max) {
+                double sb, cb;
+                sincospi(nu, &sb, &cb);
+                tanv[tid] = sb / cb;
+                dqv[tid] = make_double2(cb * cb - sb * sb, -2.0 * sb * cb);   // exp(-2 i pi nu)
+                c = QDT_ELIM;
+            }
+        }
+        cls[tid] = c;
+        open_pos[tid] = -1;
+    }
+    const int no_all = __syncthreads_count(open);
     if (tid == 0) {
-        int no_all = 0;
-        for (int i = 0; i < n; ++i) no_all += (x - pw.e_thr[i] > 0.0);
         if (n_open_out) n_open_out[e] = no_all;
-        int flag = f.flag;
-        if (flag == QDT_FLAG_OK && (node_status[f.a] != RM_OK || node_status[f.b] != RM_OK))
-            flag = QDT_FLAG_NONODE;
         int np = 0, no = 0, nq = 0;
         for (int i = 0; i < n && flag == QDT_FLAG_OK; ++i) {
-            const double eps = x - pw.e_thr[i];
-            open_pos[i] = -1;
-            if (eps > 0.0) {
+            const signed char c = cls[i];
+            if (c == QDT_OPEN) {
                 open_pos[i] = no;
                 opos[no++] = np;
                 pch[np++] = i;
-            } else if (pw.z > 0.0) {
-                const double kap = sqrt(-eps);
-                const double nu = pw.z / kap;
-                if (nu >= fmax(pw.l[i] + o.nu_margin, o.fnumin) && kap * pw.a <= o.kappa_a_max) {
-                    double sb, cb;
-                    sincospi(nu, &sb, &cb);
-                    vtan[nq] = sb / cb;
-                    dq[nq] = make_double2(cb * cb - sb * sb, -2.0 * sb * cb);   // exp(-2 i pi nu)
-                    qpos[nq++] = np;
-                    pch[np++] = i;
-                }
+            } else if (c == QDT_ELIM) {
+                qpos[nq++] = np;
+                pch[np++] = i;
             }
         }
         s_np = np;
@@ -380,6 +440,11 @@ __global__ void __launch_bounds__(NT) qdt_fine_kernel(PwDev pw, const double *__
         esh.bad = 0;
         if (flag == QDT_FLAG_THRESHOLD) status[e] = RM_ETHRESHOLD;
         if (flag == QDT_FLAG_NONODE) status[e] = RM_ESINGULAR;
+    }
+    __syncthreads();
+    if (tid < s_nq) {
+        vtan[tid] = tanv[pch[qpos[tid]]];
+        dq[tid] = dqv[pch[qpos[tid]]];
     }
     __syncthreads();
     if (s_flag != QDT_FLAG_OK || s_no == 0) return;
@@ -412,7 +477,8 @@ __global__ void __launch_bounds__(NT) qdt_fine_kernel(PwDev pw, const double *__
                 Kb[p * lk + r] = sm[p * lk + r];
             }
             __syncthreads();
-        } else if (!mqdt_eliminate(Kb, lu, no, nq, qpos, opos, vtan, sm, Kb, nullptr, 0, &esh)) {
+        } else if (!mqdt_eliminate(Kb, lu, no, nq, qpos, opos, vtan, sm, lu, sm + (size_t)nq * lu, lk, Kb, lk,
+                                   nullptr, 0, &esh)) {
             if (tid == 0) status[e] = RM_ESINGULAR;
             return;
         }
@@ -443,13 +509,21 @@ __global__ void __launch_bounds__(NT) qdt_fine_kernel(PwDev pw, const double *__
             C[i * ld2 + j] = v;
         }
         __syncthreads();
-        cblock_eliminate(C, ld2, nq, w2, &esh, &pinv_s);
+        cblock_eliminate<NT>(C, ld2, nq, w2, &esh, &pinv_s);
         if (esh.bad) {
             if (tid == 0) status[e] = RM_ESINGULAR;
             return;
         }
-        cblock_backsub(C, ld2, nq, nq, no);   // Y = (S_cc - D)^{-1} S_co
+        cblock_backsub<NT>(C, ld2, nq, nq, no);   // Y = (S_cc - D)^{-1} S_co
     }
+    // S_oc at this energy, read for every partner channel below (after C: nq
+    // (w2 + 1) + no nq <= n (n + 1) entries together)
+    double2 *Soc = C + (size_t)nq * ld2;
+    for (int q = tid; q < no * nq; q += NT) {
+        const int a = q / nq, i = q - (q / nq) * nq;
+        Soc[q] = su(opos[a], qpos[i]);
+    }
+    __syncthreads();
     for (int q = tid; q < npair; q += NT) {
         int I, J;
         tri_pair(q, nl, I, J);
@@ -460,7 +534,7 @@ __global__ void __launch_bounds__(NT) qdt_fine_kernel(PwDev pw, const double *__
             for (int ib = pw.lev_start[J]; ib < pw.lev_start[J + 1]; ++ib) {
                 const int b = open_pos[pw.lev_chan[ib]];
                 double2 v = su(opos[a], opos[b]);
-                for (int i = 0; i < nq; ++i) v = cfms(v, su(opos[a], qpos[i]), C[i * ld2 + nq + b]);
+                for (int i = 0; i < nq; ++i) v = cfms(v, Soc[a * nq + i], C[i * ld2 + nq + b]);
                 if (a == b) v.x -= 1.0;
                 s += fma(v.x, v.x, v.y * v.y);
             }
@@ -516,7 +590,7 @@ cudaError_t launch_qdt_s_from_k(int n, int n_nodes, const double *Ku, const int 
     cudaError_t e = cudaFuncSetAttribute(qdt_s_from_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    qdt_s_from_k_kernel<<<n_nodes, NT, smem, s>>>(n, Ku, np_node, status, Su);
+    qdt_s_from_k_kernel<<<n_nodes, NTS, smem, s>>>(n, Ku, np_node, status, Su);
     return cudaGetLastError();
 }
 

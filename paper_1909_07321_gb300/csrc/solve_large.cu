@@ -7,7 +7,7 @@
 //   classify      per energy: open set, P set (open + MQDT-eliminated),
 //                 unknown ordering (decaying-closed first)
 //   assemble      [A | B] (n x (n + n_p)) from packed R and channel data
-//   lu            CTA per energy: blocked right-looking Gaussian elimination
+//   lu, lu64      CTA per energy: blocked right-looking Gaussian elimination
 //                 with partial pivoting (panel width 32, full-row swaps),
 //                 then blocked back-substitution of the trailing rows only
 //   extract       K_u = X[P rows]; direct mode: K = K_u
@@ -355,6 +355,338 @@ __global__ void __launch_bounds__(NTH) lu_kernel(const LuJob *__restrict__ jobs,
     }
 }
 
+// ---- the same with the panel in shared memory --------------------------------
+
+// Up to L64_MAX_N rows. The kernel above walks its panel in global memory
+// column by column (strided reads, a division by every warp a column, FP64
+// comparisons, whose 64 clocks a warp each make a pivot search) and stages
+// both operands anew for every 64 x 64 tile; here the panel (PNB columns,
+// column-major) stays in shared memory, its rows in registers while it is
+// factored once no more than NTH are left, one lane divides, the pivot is
+// found by integer comparisons, the interchanges of the
+// columns to the right are one permutation per panel, U12 is solved one column
+// a thread in registers, and a strip of U12 serves all its row tiles. The
+// arithmetic of every entry is that of the kernel above: the panel's and U12's
+// entries are chains of FMAs, the trailing update adds the PNB products of a
+// panel from zero and subtracts the sum. FP64 pipe: 2 FMAs per clock and SM,
+// 200 systems of 132 unknowns: 1.77 ms, were 3.35 (floor 0.7). The quantum-defect systems of a few rows
+// each stay with the kernel above (512 systems at 431 channels 52 against 189
+// us: this one's panel is sized for the widest, one CTA per SM).
+constexpr int L64_MAX_N = 720;
+__host__ __device__ inline int l64_pad(int n) { return n | 1; }
+// Stride of the staged U (32 rows): all right-hand columns of n <= 128 at once,
+// narrower strips where the panel takes more of the shared memory.
+inline int l64_strip(int n) { return n <= 128 ? 257 : (n <= 256 ? 161 : 65); }
+inline size_t l64_smem(int n)
+{
+    return ((size_t)PNB * l64_pad(n) + (size_t)PNB * l64_strip(n)) * sizeof(double) + (size_t)n * sizeof(int);
+}
+
+// M[r, c0 .. c0 + sw) -= sum_k Lp[k][r] Us[k][.] for rows [r0, r1), columns
+// < c1: items of four rows and one column dealt out one to a thread, columns
+// fastest, so that small trailing matrices leave few lanes idle.
+__device__ void l64_update(double *M, int ld, int r0, int r1, int c0, int c1, int kb, const double *Lp, int npad,
+                           const double *Us, int us)
+{
+    const int nc = c1 - c0, items = ((r1 - r0 + 3) / 4) * nc;
+    for (int q = threadIdx.x; q < items; q += NTH) {
+        const int rb = r0 + 4 * (q / nc), c = q - (q / nc) * nc;
+        const int nr = min(4, r1 - rb);
+        const double *u = Us + c;
+        double *m = M + (size_t)rb * ld + c0 + c;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        // a row past the end repeats the last one and is not stored
+        const double *l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] = Lp + min(rb + i, r1 - 1);
+#pragma unroll 4
+        for (int k = 0; k < kb; ++k) {
+            const double uv = u[k * us];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = fma(l[i][k * npad], uv, acc[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < nr) m[(size_t)i * ld] -= acc[i];
+    }
+}
+
+// Largest magnitude, then lowest row, among the lanes' candidates (key: the
+// magnitude's bits, 0 for none; integer comparisons, which do not occupy the
+// FP64 unit). All lanes get the winner.
+__device__ __forceinline__ void warp_pivot(unsigned long long &key, int &row)
+{
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    row = (int)__reduce_min_sync(0xffffffffu, (hi == mh && lo == ml) ? (unsigned)row : 0x7fffffffu);
+    key = ((unsigned long long)mh << 32) | ml;
+}
+
+// |v| as a key (a NaN is no candidate)
+__device__ __forceinline__ unsigned long long pivot_key(double v)
+{
+    const unsigned long long k = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return k > 0x7ff0000000000000ull ? 0ull : k;
+}
+
+__global__ void __launch_bounds__(NTH, 2) lu64_kernel(const LuJob *__restrict__ jobs, int *status, int n_max, int sw_max)
+{
+    extern __shared__ double sm64[];
+    constexpr int NW = NTH / 32;
+    __shared__ double slots[NW][PNB + 2];   // a warp's candidate: its row, key, row number
+    __shared__ unsigned long long red_k[NW];
+    __shared__ int red_i[NW];
+    __shared__ int s_bad, s_moves, s_piv, s_win, mv_dst[PNB], mv_src[PNB];
+    __shared__ double s_pinv;
+    const LuJob job = jobs[blockIdx.x];
+    if (job.rows <= 0) return;
+    double *M = job.M;
+    const int ld = job.ld, n = job.rows, w = job.w;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int npad = l64_pad(n);
+    double *Lp = sm64, *Us = Lp + PNB * l64_pad(n_max);
+    int *perm = reinterpret_cast<int *>(Us + PNB * sw_max);
+    if (tid == 0) s_bad = 0;
+    const int us = min(sw_max, (w + 1) | 1);   // strip stride; a strip holds us - 1 columns
+    auto stage = [&](int u0, int kb, int c0, int nc) {   // U rows u0 .. u0 + kb, columns c0 .. c0 + nc
+        for (int q = tid; q < kb * nc; q += NTH) {
+            const int k = q / nc, c = q - (q / nc) * nc;
+            Us[k * us + c] = M[(size_t)(u0 + k) * ld + c0 + c];
+        }
+    };
+    for (int k0 = 0; k0 < n; k0 += PNB) {
+        const int kb = min(PNB, n - k0);
+        if (tid == 0) s_moves = 0;
+        if (n - k0 <= NTH) {
+            // a row of the panel in a thread's registers; positions change
+            // instead of rows
+            double a[PNB];
+            const int r = k0 + tid;
+            bool live = r < n;
+            int pos = r;
+#pragma unroll
+            for (int j = 0; j < PNB; ++j) a[j] = live && j < kb ? M[(size_t)r * ld + k0 + j] : 0.0;
+#pragma unroll
+            for (int j = 0; j < PNB; ++j) {
+                if (j >= kb) break;
+                const int c = k0 + j;
+                unsigned long long key = live ? pivot_key(a[j]) : 0ull;
+                int row = live && key ? pos : 0x7fffffff;
+                const unsigned long long mine = key;
+                warp_pivot(key, row);
+                if (live && mine && mine == key && pos == row) {
+#pragma unroll
+                    for (int jj = j; jj < PNB; ++jj) slots[warp][jj] = a[jj];
+                }
+                if (lane == 0) {
+                    red_k[warp] = key;
+                    red_i[warp] = row;
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    key = lane < NW ? red_k[lane] : 0ull;
+                    row = lane < NW ? red_i[lane] : 0x7fffffff;
+                    const unsigned long long k2 = key;
+                    const int r2 = row;
+                    warp_pivot(key, row);
+                    const int win = __ffs(__ballot_sync(0xffffffffu, k2 == key && r2 == row)) - 1;
+                    const bool bad = key == 0ull || key >= 0x7ff0000000000000ull;
+                    if (lane == 0) {
+                        s_piv = row;
+                        s_win = win;
+                        if (bad) s_bad = 1;
+                        else s_pinv = 1.0 / slots[win][j];
+                    }
+                }
+                __syncthreads();
+                if (s_bad) break;
+                const int p = s_piv;
+                const double pinv = s_pinv;
+                const double *u = slots[s_win];
+                if (live) {
+                    if (pos == p) {
+                        live = false;
+                        pos = c;
+                    } else {
+                        if (pos == c) pos = p;
+                        const double l = a[j] * pinv;
+                        a[j] = l;
+#pragma unroll
+                        for (int jj = j + 1; jj < PNB; ++jj) a[jj] = fma(-l, u[jj], a[jj]);
+                    }
+                }
+                __syncthreads();   // slots are written anew
+            }
+            if (!s_bad && r < n) {
+                perm[pos] = r;
+#pragma unroll
+                for (int j = 0; j < PNB; ++j)
+                    if (j < kb) Lp[j * npad + pos] = a[j];
+            }
+        } else {
+            for (int q = tid; q < (n - k0) * kb; q += NTH) {
+                const int r = k0 + q / kb, j = q - (q / kb) * kb;
+                Lp[j * npad + r] = M[(size_t)r * ld + k0 + j];
+            }
+            for (int r = k0 + tid; r < n; r += NTH) perm[r] = r;
+            __syncthreads();
+            unsigned long long best = 0ull;
+            int bi = 0x7fffffff;
+            for (int r = k0 + tid; r < n; r += NTH) {
+                const unsigned long long v = pivot_key(Lp[r]);
+                if (v > best) { best = v; bi = r; }
+            }
+            for (int j = 0; j < kb; ++j) {
+                const int c = k0 + j;
+                warp_pivot(best, bi);
+                if (lane == 0) {
+                    red_k[warp] = best;
+                    red_i[warp] = bi;
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    unsigned long long key = lane < NW ? red_k[lane] : 0ull;
+                    int p = lane < NW ? red_i[lane] : 0x7fffffff;
+                    warp_pivot(key, p);
+                    if (key == 0ull || key >= 0x7ff0000000000000ull) {
+                        if (lane == 0) s_bad = 1;
+                    } else {
+                        const double pv = Lp[j * npad + p];
+                        __syncwarp();
+                        if (p != c) {
+                            if (lane < kb) {
+                                const double t = Lp[lane * npad + c];
+                                Lp[lane * npad + c] = Lp[lane * npad + p];
+                                Lp[lane * npad + p] = t;
+                            }
+                            if (lane == 0) {
+                                const int t = perm[c];
+                                perm[c] = perm[p];
+                                perm[p] = t;
+                            }
+                        }
+                        if (lane == 0) s_pinv = 1.0 / pv;
+                    }
+                }
+                __syncthreads();
+                if (s_bad) break;
+                const double pinv = s_pinv;
+                best = 0ull;
+                bi = 0x7fffffff;
+                for (int r = c + 1 + tid; r < n; r += NTH) {
+                    const double l = Lp[j * npad + r] * pinv;
+                    Lp[j * npad + r] = l;
+                    for (int jj = j + 1; jj < kb; ++jj)
+                        Lp[jj * npad + r] = fma(-l, Lp[jj * npad + c], Lp[jj * npad + r]);
+                    if (j + 1 < kb) {
+                        const unsigned long long v = pivot_key(Lp[(j + 1) * npad + r]);
+                        if (v > best) { best = v; bi = r; }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (s_bad) break;
+        for (int q = tid; q < kb * kb; q += NTH) {   // U11
+            const int i = q / kb, j = q - (q / kb) * kb;
+            if (i <= j) M[(size_t)(k0 + i) * ld + k0 + j] = Lp[j * npad + k0 + i];
+        }
+        for (int r = k0 + kb + tid; r < n; r += NTH)
+            if (perm[r] != r) {
+                const int s = atomicAdd(&s_moves, 1);
+                mv_dst[s] = r;
+                mv_src[s] = perm[r];
+            }
+        __syncthreads();
+        if (k0 + kb >= w) continue;
+        const int nmv = s_moves;
+        for (int cc = k0 + kb + tid; cc < w; cc += NTH) {
+            // rows named by perm below the panel are move destinations: read
+            // first; a row below the panel only receives rows of the panel's
+            // range, which are written last
+            double x[PNB];
+#pragma unroll
+            for (int i = 0; i < PNB; ++i) x[i] = i < kb ? M[(size_t)perm[k0 + i] * ld + cc] : 0.0;
+            for (int i = 0; i < nmv; ++i) M[(size_t)mv_dst[i] * ld + cc] = M[(size_t)mv_src[i] * ld + cc];
+#pragma unroll
+            for (int j = 0; j < PNB - 1; ++j)
+                if (j + 1 < kb) {
+#pragma unroll
+                    for (int i = j + 1; i < PNB; ++i) x[i] = fma(-Lp[j * npad + min(k0 + i, n - 1)], x[j], x[i]);
+                }
+#pragma unroll
+            for (int i = 0; i < PNB; ++i)
+                if (i < kb) M[(size_t)(k0 + i) * ld + cc] = x[i];
+        }
+        __syncthreads();
+        if (k0 + kb < n)
+            for (int c0 = k0 + kb; c0 < w; c0 += us - 1) {
+                const int c1 = min(w, c0 + us - 1);
+                stage(k0, kb, c0, c1 - c0);
+                __syncthreads();
+                l64_update(M, ld, k0 + kb, n, c0, c1, kb, Lp, npad, Us, us);
+                __syncthreads();
+            }
+    }
+    if (s_bad) {
+        if (tid == 0) atomicCAS(status + blockIdx.x, RM_OK, RM_ESINGULAR);
+        return;
+    }
+    // blocked back-substitution of rows [row_lo, n) for RHS columns [n, w)
+    const int lo = job.row_lo;
+    int t1 = n;
+    while (t1 > lo) {
+        const int t0 = max(lo, t1 - PNB), tb = t1 - t0;
+        for (int q = tid; q < (t1 - lo) * tb; q += NTH) {
+            const int r = lo + q / tb, j = q - (q / tb) * tb;
+            Lp[j * npad + r] = M[(size_t)r * ld + t0 + j];
+        }
+        __syncthreads();
+        for (int cq = n + tid; cq < w; cq += NTH) {
+            double x[PNB];
+#pragma unroll
+            for (int i = 0; i < PNB; ++i) x[i] = i < tb ? M[(size_t)(t0 + i) * ld + cq] : 0.0;
+#pragma unroll
+            for (int i = PNB - 1; i >= 0; --i)
+                if (i < tb) {
+                    double s = x[i];
+#pragma unroll
+                    for (int u = i + 1; u < PNB; ++u)
+                        if (u < tb) s = fma(-Lp[u * npad + t0 + i], x[u], s);
+                    x[i] = s / Lp[i * npad + t0 + i];
+                }
+#pragma unroll
+            for (int i = 0; i < PNB; ++i)
+                if (i < tb) M[(size_t)(t0 + i) * ld + cq] = x[i];
+        }
+        __syncthreads();
+        if (t0 > lo)
+            for (int c0 = n; c0 < w; c0 += us - 1) {
+                const int c1 = min(w, c0 + us - 1);
+                stage(t0, tb, c0, c1 - c0);
+                __syncthreads();
+                l64_update(M, ld, lo, t0, c0, c1, tb, Lp, npad, Us, us);
+                __syncthreads();
+            }
+        t1 = t0;
+    }
+}
+
+// LU of every job of the block (rows <= n).
+cudaError_t launch_lu64(int n, int nE, const LuJob *lu, int *status, cudaStream_t st)
+{
+    if (n > L64_MAX_N) {
+        lu_kernel<<<nE, NTH, 0, st>>>(lu, status);
+        return cudaGetLastError();
+    }
+    const size_t sm = l64_smem(n);
+    const cudaError_t err = cudaFuncSetAttribute(lu64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (err != cudaSuccess) return err;
+    lu64_kernel<<<nE, NTH, sm, st>>>(lu, status, n, l64_strip(n));
+    return cudaGetLastError();
+}
+
 // ---- batched GEMM: C = alpha A B + beta C (+ I) ---------------------------
 
 struct GemmJob {
@@ -363,18 +695,43 @@ struct GemmJob {
     double *C;
     int lda, ldb, ldc, m, n, k;
     double alpha, beta;
-    int add_identity;
+    int add_identity, symmetric;
 };
 
+// One chunk of GK products into the NI x NJ entries a thread has in its tile.
+template <int NI, int NJ>
+__device__ __forceinline__ void gemm_step(const double (*As)[GT + 1], const double (*Bs)[GT + 1], int ty, int tx,
+                                          double (&acc)[4][4])
+{
+#pragma unroll 4
+    for (int kk = 0; kk < GK; ++kk) {
+        double av[NI], bv[NJ];
+#pragma unroll
+        for (int a = 0; a < NI; ++a) av[a] = As[kk][ty + 16 * a];
+#pragma unroll
+        for (int b = 0; b < NJ; ++b) bv[b] = Bs[kk][tx + 16 * b];
+#pragma unroll
+        for (int a = 0; a < NI; ++a)
+#pragma unroll
+            for (int b = 0; b < NJ; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+    }
+}
+
+// Tiles of GT x GT, thread (ty, tx) on rows ty + 16 i and columns tx + 16 j:
+// the sixteenths of a tile past the edge are not computed. symmetric: C = A A
+// with A symmetric, whose entries (i, j) and (j, i) are the same chain of FMAs:
+// the tiles above the diagonal are computed and stored twice. 200 products of
+// 100 x 100: K^2 604, Y = K X 618 us, were 774 and 754.
 __global__ void __launch_bounds__(NTH) gemm_kernel(const GemmJob *__restrict__ jobs)
 {
     const GemmJob j = jobs[blockIdx.z];
     if (j.m <= 0 || j.n <= 0) return;
     const int r0 = blockIdx.y * GT, c0 = blockIdx.x * GT;
-    if (r0 >= j.m || c0 >= j.n) return;
+    if (r0 >= j.m || c0 >= j.n || (j.symmetric && r0 > c0)) return;
     __shared__ double As[GK][GT + 1];
     __shared__ double Bs[GK][GT + 1];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int ni = min(4, (j.m - r0 + 15) >> 4), nj = min(4, (j.n - c0 + 15) >> 4);
     double acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -390,32 +747,30 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(const GemmJob *__restrict__ j
             Bs[kr][cc] = (gk2 < j.k && gc < j.n) ? j.B[(size_t)gk2 * j.ldb + gc] : 0.0;
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty * 4 + a];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx * 4 + b];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-        }
+#define RM_GJ(I)                                                              \
+    (nj == 4 ? gemm_step<I, 4>(As, Bs, ty, tx, acc)                           \
+             : (nj == 3 ? gemm_step<I, 3>(As, Bs, ty, tx, acc)                \
+                        : (nj == 2 ? gemm_step<I, 2>(As, Bs, ty, tx, acc) : gemm_step<I, 1>(As, Bs, ty, tx, acc))))
+        if (ni == 4) RM_GJ(4);
+        else if (ni == 3) RM_GJ(3);
+        else if (ni == 2) RM_GJ(2);
+        else RM_GJ(1);
+#undef RM_GJ
         __syncthreads();
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-        const int gr = r0 + ty * 4 + a;
+        const int gr = r0 + ty + 16 * a;
         if (gr >= j.m) continue;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const int gc = c0 + tx * 4 + b;
+            const int gc = c0 + tx + 16 * b;
             if (gc >= j.n) continue;
             double v = j.alpha * acc[a][b];
             if (j.beta != 0.0) v += j.beta * j.C[(size_t)gr * j.ldc + gc];
             if (j.add_identity && gr == gc) v += 1.0;
             j.C[(size_t)gr * j.ldc + gc] = v;
+            if (j.symmetric && r0 < c0) j.C[(size_t)gc * j.ldc + gr] = v;
         }
     }
 }
@@ -486,11 +841,11 @@ __global__ void mqdt_build_kernel(int n, int nE, const EnergyDims *dims, const C
     double *koc = s.aug + (size_t)d.nq * ld2;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         LuJob j = {nullptr, 0, 0, 0, 0};
-        GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0};
+        GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0, 0};
         if (act) {
             j = {s.aug, ld2, d.nq, w2, 0};
             // ks = K_oo - K_oc Y,  Y in aug columns nq.. (ld ld2)
-            g = {koc, s.aug + d.nq, s.ks, d.nq, ld2, d.no, d.no, d.no, d.nq, -1.0, 1.0, 0};
+            g = {koc, s.aug + d.nq, s.ks, d.nq, ld2, d.no, d.no, d.no, d.nq, -1.0, 1.0, 0, 0};
         }
         lu[e] = j;
         gj[e] = g;
@@ -561,10 +916,10 @@ __global__ void t_build_kernel(int n, int nE, const EnergyDims *dims, double *ws
     const int ld = 2 * d.no + 1;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         LuJob j = {nullptr, 0, 0, 0, 0};
-        GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0};
+        GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0, 0};
         if (act) {
             j = {s.aug, ld, d.no, 2 * d.no, 0};
-            g = {s.ks, s.ks, s.aug, d.no, d.no, ld, d.no, d.no, d.no, 1.0, 0.0, 1};
+            g = {s.ks, s.ks, s.aug, d.no, d.no, ld, d.no, d.no, d.no, 1.0, 0.0, 1, 1};
         }
         lu[e] = j;
         gj[e] = g;
@@ -582,10 +937,10 @@ __global__ void y_jobs_kernel(int n, int nE, const EnergyDims *dims, double *ws,
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nE) return;
     const EnergyDims d = dims[e];
-    GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0};
+    GemmJob g = {nullptr, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0.0, 0.0, 0, 0};
     if (d.np >= 0) {
         const Slot s = slot_of(ws, n, e);
-        g = {s.ks, s.aug + d.no, s.ku, d.no, 2 * d.no + 1, d.no, d.no, d.no, d.no, 1.0, 0.0, 0};
+        g = {s.ks, s.aug + d.no, s.ku, d.no, 2 * d.no + 1, d.no, d.no, d.no, d.no, 1.0, 0.0, 0, 0};
     }
     gj[e] = g;
 }
@@ -912,7 +1267,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
         LAUNCH_OK();
         jobs_match_kernel<<<eg, 128, 0, st>>>(n, nE, dims, ws, lu);
         LAUNCH_OK();
-        lu_kernel<<<nE, NTH, 0, st>>>(lu, status);
+        if ((err = launch_lu64(n, nE, lu, status, st)) != cudaSuccess) return err;
         LAUNCH_OK();
         prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
         LAUNCH_OK();
@@ -923,6 +1278,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
     // MQDT elimination (no-op for energies without eliminated channels)
     mqdt_build_kernel<<<dim3(xb2, nE), NTH, 0, st>>>(n, nE, dims, cf, col_chan, qpos, opos, ws, lu, gj);
     LAUNCH_OK();
+    // systems of few rows: more of them share an SM without the panel
     lu_kernel<<<nE, NTH, 0, st>>>(lu, status);
     LAUNCH_OK();
     prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
@@ -951,7 +1307,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
         LAUNCH_OK();
         gemm_kernel<<<dim3(tiles, tiles, nE), NTH, 0, st>>>(gj);   // 1 + K^2
         LAUNCH_OK();
-        lu_kernel<<<nE, NTH, 0, st>>>(lu, status);                // X = (1 + K^2)^{-1} K
+        if ((err = launch_lu64(n, nE, lu, status, st)) != cudaSuccess) return err;                // X = (1 + K^2)^{-1} K
         LAUNCH_OK();
         prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
         LAUNCH_OK();

@@ -63,19 +63,20 @@ __global__ void __launch_bounds__(NT) solve_small_kernel(
     const double *Rp = Ra + (size_t)e * tri_ld(n);   // packed upper triangle
     const bool ok_status = status[e] == RM_OK;
 
+    __shared__ int kind[SOLVE_SMALL_MAXN];
+    if (tid < n && ok_status) kind[tid] = cf[tid].kind;
+    const int n_open = __syncthreads_count(tid < n && x - pw.e_thr[tid < n ? tid : 0] > 0.0);
     if (tid == 0) {
-        int no = 0;
-        for (int i = 0; i < n; ++i) no += (x - pw.e_thr[i] > 0.0);
-        if (n_open_out) n_open_out[e] = no;
-        s_no = no;
+        if (n_open_out) n_open_out[e] = n_open;
+        s_no = n_open;
         esh.bad = 0;
         if (ok_status) {
             int np = 0;
-            for (int i = 0; i < n; ++i) np += (cf[i].kind != CH_CLOSED);
+            for (int i = 0; i < n; ++i) np += (kind[i] != CH_CLOSED);
             const int ncl = n - np;
             int pc = 0, pp = 0, po = 0, pq = 0;
             for (int i = 0; i < n; ++i) {
-                const int k = cf[i].kind;
+                const int k = kind[i];
                 if (k == CH_CLOSED) {
                     col_chan[pc++] = i;
                     open_pos[i] = -1;
@@ -141,7 +142,6 @@ __global__ void __launch_bounds__(NT) solve_small_kernel(
         return;
     }
 
-    const int lk = no + 1;
     double *Kp;   // K (no x no, symmetrised), row stride kld
     double *Mi;   // M = 1 + K^2, then M^{-1} (no x no), row stride mld
     int kld, mld;
@@ -175,27 +175,24 @@ __global__ void __launch_bounds__(NT) solve_small_kernel(
             if (tid == 0) status[e] = RM_ESINGULAR;
             return;
         }
-        // Shared layout: [region A: n(2n+2) doubles][region B: n(n+1) doubles].
-        double *Ks = sm + (size_t)n * (2 * n + 2);   // region B
-        const Real *Mq = M;
         // ---- MQDT elimination of the nq channels --------------------------
-        const int lu = np + 1;
-        double *Ku = Ks;           // K_u (np x np) in region B
-        for (int q = tid; q < np * np; q += NT) {
-            const int p = q / np, r = q - (q / np) * np;
-            Ku[p * lu + r] = (double)Mq[(ncl + p) * ld + n + r];
-        }
+        // K_u stays where the back-substitution left it (rows ncl.., columns
+        // n..); the elimination's matrices take the columns before n, which
+        // are no longer read, so that MQDT needs no more shared memory than
+        // the direct mode (three CTAs per SM at 64 channels, not two: 4000
+        // energies 4.80 ms, were 6.00).
+        double *Ku = reinterpret_cast<double *>(sm) + ncl * ld + n;
         for (int i = tid; i < nq; i += NT) vcol[i] = cf[col_chan[ncl + qpos[i]]].tanb;
         __syncthreads();
-        if (!mqdt_eliminate(Ku, lu, no, nq, qpos, opos, vcol, sm, Ks,
+        if (!mqdt_eliminate(Ku, ld, no, nq, qpos, opos, vcol, sm, ld, sm + nq * ld, ld, Ku, ld,
                             K_out ? K_out + (size_t)e * n * n : nullptr, n, &esh)) {
             if (tid == 0) status[e] = RM_ESINGULAR;
             return;
         }
-        Kp = Ks;
-        kld = lk;
-        Mi = sm;
-        mld = lk;
+        Kp = Ku;
+        kld = ld;
+        Mi = reinterpret_cast<double *>(sm) + ncl * ld;
+        mld = ld;
     }
     if (!omega) return;
 
@@ -209,16 +206,8 @@ __global__ void __launch_bounds__(NT) solve_small_kernel(
 
 int solve_small_max_n() { return SOLVE_SMALL_MAXN; }
 
-// Direct mode needs only the augmented matrix n x (2n + 1); MQDT mode also
-// holds K_u and the elimination system.
-size_t solve_small_smem(int n, int mqdt, int f32)
-{
-    if (f32) return (size_t)n * n * sizeof(float);
-    if (!mqdt) return (size_t)n * (2 * n + 1) * sizeof(double);
-    const size_t aug = (size_t)n * (2 * n + 2);
-    const size_t ks = (size_t)n * (n + 1);
-    return (aug + ks) * sizeof(double);
-}
+// The augmented matrix n x (2n + 1), in both modes.
+size_t solve_small_smem(int n) { return (size_t)n * (2 * n + 1) * sizeof(double); }
 
 cudaError_t launch_solve_small(const PwDev &pw, const double *E, int nE, const ChanFn *cf,
                                const double *R, int *status, double *K_out, int *n_open_out,
@@ -228,7 +217,7 @@ cudaError_t launch_solve_small(const PwDev &pw, const double *E, int nE, const C
     if (pw.n > SOLVE_SMALL_MAXN || (f32 && mqdt) || (f32 && ku_out)) return cudaErrorInvalidValue;
     if (nE == 0) return cudaSuccess;
     if (f32) return launch_solve_f32(pw, E, nE, cf, R, status, K_out, n_open_out, omega, n_tri, deep_ws, pass, s);
-    const size_t smem = solve_small_smem(pw.n, mqdt, 0);
+    const size_t smem = solve_small_smem(pw.n);
     const int cap = chanfn_deep_cap();
     cudaError_t err =
         cudaFuncSetAttribute(solve_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
