@@ -29,7 +29,7 @@
 //   mqdt          as above (FP64)
 //   zbuild        Z = 1 - iK (FP32 complex)
 //   zsweep        Z -> -(1 - iK)^{-1};  T = 2 (1 - iK)^{-1} - 2
-//   t2z           |T_ab|^2 = 4 |Z_ab + delta_ab|^2 (symmetrised, FP64)
+//   omega_z       as omega, |T_ab|^2 = 4 |Z_ab + delta_ab|^2 (FP64) formed there
 //
 // Per-energy sizes differ (n_o, n_p vary with E); every kernel reads them from
 // the per-energy descriptors and idles outside them.
@@ -61,49 +61,63 @@ struct EnergyDims {
 
 // ---- classify -----------------------------------------------------------
 
+// A warp per energy, 32 channels at a time (one thread's walk over 1000
+// channels took 477 us for 256 energies).
 __global__ void classify_kernel(PwDev pw, const double *__restrict__ E, int nE,
                                 const ChanFn *__restrict__ cfa, const int *__restrict__ status,
                                 EnergyDims *dims, int *col_chan, int *open_pos, int *qpos,
                                 int *opos, int *n_open_out)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= nE) return;
     const int n = pw.n;
     const double x = E[e];
-    int no = 0;
-    for (int i = 0; i < n; ++i) no += (x - pw.e_thr[i] > 0.0);
-    if (n_open_out) n_open_out[e] = no;
+    const bool ok = status[e] == RM_OK;
+    const ChanFn *cf = cfa + (size_t)e * n;
+    int no = 0, np = 0;
+    for (int b = 0; b < n; b += 32) {
+        const int i = b + lane;
+        no += __popc(__ballot_sync(0xffffffffu, i < n && x - pw.e_thr[i < n ? i : 0] > 0.0));
+        if (ok) np += __popc(__ballot_sync(0xffffffffu, i < n && cf[i < n ? i : 0].kind != CH_CLOSED));
+    }
+    if (lane == 0 && n_open_out) n_open_out[e] = no;
     EnergyDims d = {no, -1, 0, 0};
-    if (status[e] == RM_OK && no > 0) {
-        const ChanFn *cf = cfa + (size_t)e * n;
-        int np = 0;
-        for (int i = 0; i < n; ++i) np += (cf[i].kind != CH_CLOSED);
+    if (ok && no > 0) {
         const int ncl = n - np;
-        int pc = 0, pp = 0, po = 0, pq = 0;
+        int pc = 0, po = 0, pq = 0;
         int *cc = col_chan + (size_t)e * n, *op = open_pos + (size_t)e * n;
         int *qp = qpos + (size_t)e * n, *oq = opos + (size_t)e * n;
-        for (int i = 0; i < n; ++i) {
-            const int k = cf[i].kind;
+        const unsigned below = (1u << lane) - 1u;
+        for (int b = 0; b < n; b += 32) {
+            const int i = b + lane;
+            const int k = i < n ? cf[i].kind : -1;
+            const unsigned mc = __ballot_sync(0xffffffffu, k == CH_CLOSED);
+            const unsigned mo = __ballot_sync(0xffffffffu, k == CH_OPEN);
+            const unsigned mq = __ballot_sync(0xffffffffu, k >= 0 && k != CH_CLOSED && k != CH_OPEN);
             if (k == CH_CLOSED) {
-                cc[pc++] = i;
+                cc[pc + __popc(mc & below)] = i;
                 op[i] = -1;
-            } else {
+            } else if (k >= 0) {
+                const int pp = po + pq + __popc((mo | mq) & below);
                 cc[ncl + pp] = i;
                 if (k == CH_OPEN) {
-                    op[i] = po;
-                    oq[po++] = pp;
+                    const int o = po + __popc(mo & below);
+                    op[i] = o;
+                    oq[o] = pp;
                 } else {
                     op[i] = -1;
-                    qp[pq++] = pp;
+                    qp[pq + __popc(mq & below)] = pp;
                 }
-                ++pp;
             }
+            pc += __popc(mc);
+            po += __popc(mo);
+            pq += __popc(mq);
         }
         d.np = np;
         d.nq = pq;
         d.ncl = ncl;
     }
-    dims[e] = d;
+    if (lane == 0) dims[e] = d;
 }
 
 // ---- CTA order of the per-energy FP32 kernels ------------------------------
@@ -961,6 +975,18 @@ __global__ void t2_kernel(int n, int nE, const EnergyDims *dims, double *ws)
     }
 }
 
+// Level pair q (row-wise upper triangle of nl levels).
+__device__ __forceinline__ void level_pair(int q, int nl, int &I, int &J)
+{
+    const float t = (float)(2 * nl + 1);
+    int p = (int)((t - sqrtf(fmaxf(t * t - 8.0f * (float)q, 0.0f))) * 0.5f);
+    p = min(max(p, 0), nl - 1);
+    while (p > 0 && tri_idx(p, p, nl) > q) --p;
+    while (p + 1 < nl && tri_idx(p + 1, p + 1, nl) <= q) ++p;
+    I = p;
+    J = p + (q - tri_idx(p, p, nl));
+}
+
 __global__ void omega_kernel(PwDev pw, const double *__restrict__ E, int nE,
                              const EnergyDims *__restrict__ dims, const int *__restrict__ open_pos,
                              double *ws, double *omega, int n_tri)
@@ -975,9 +1001,8 @@ __global__ void omega_kernel(PwDev pw, const double *__restrict__ E, int nE,
     double *om = omega + (size_t)e * n_tri;
     const int npair = nl * (nl + 1) / 2;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < npair; q += gridDim.x * blockDim.x) {
-        int I = 0, rem = q;
-        while (rem >= nl - I) { rem -= nl - I; ++I; }
-        const int J = I + rem;
+        int I, J;
+        level_pair(q, nl, I, J);
         if (!(x - pw.lev_thr[I] > 0.0) || !(x - pw.lev_thr[J] > 0.0)) continue;
         double sum = 0.0;
         for (int ia = pw.lev_start[I]; ia < pw.lev_start[I + 1]; ++ia) {
@@ -993,37 +1018,78 @@ __global__ void omega_kernel(PwDev pw, const double *__restrict__ E, int nE,
 
 // ---- FP32 path ---------------------------------------------------------------
 
+// (float)v without the FP64 unit: round to nearest even on the bits where the
+// result is a normal float, the conversion instruction elsewhere.
+__device__ __forceinline__ float to_float(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned mh = hi & 0x7fffffffu;
+    // 2^-126 <= |v| < 2^127
+    if (mh - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)v;
+    const unsigned t = ((mh - 0x38000000u) << 3) | (lo >> 29);   // exponent and 23 bits
+    const unsigned rest = lo << 3;                                // the bits below
+    const unsigned up = (rest > 0x80000000u || (rest == 0x80000000u && (t & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (t + up));
+}
+
 // [A | 0 | B] in FP32: A = diag(Ghat) - R diag(a Ghat' - b Ghat), B as in
-// assemble_kernel, right-hand sides from column rhs0(n), zero padding.
-__global__ void assemble_f32_kernel(PwDev pw, int nE, const ChanFn *__restrict__ cfa,
-                                    const double *__restrict__ Ra, const EnergyDims *__restrict__ dims,
-                                    const int *__restrict__ col_chan, double *ws)
+// assemble_kernel, right-hand sides from column rhs0(n), zero padding. A CTA
+// takes 32 rows of one energy, 32 columns at a time: a column's factor is
+// formed once, and the entries below the diagonal, which are neighbours along
+// the rows of the packed triangle, come through shared memory. 256 energies of
+// 1000 channels: 2.62 ms, were 3.98 with a factor and a strided read per entry.
+__global__ void __launch_bounds__(256) assemble_f32_kernel(PwDev pw, int nE, const ChanFn *__restrict__ cfa,
+                                                           const double *__restrict__ Ra,
+                                                           const EnergyDims *__restrict__ dims,
+                                                           const int *__restrict__ col_chan, double *ws)
 {
     const int e = blockIdx.y;
     const EnergyDims d = dims[e];
     if (d.np < 0) return;
+    __shared__ double tr[32][33], fac[32], dia[32];
+    __shared__ int chan[32];   // -1: a zero column
     const int n = pw.n, rhs = f32d::rhs0(n), ld = f32d::aug_ld(n, d.np);
     float *M = reinterpret_cast<float *>(slot_of(ws, n, e).aug);
     const ChanFn *cf = cfa + (size_t)e * n;
     const double *Rp = Ra + (size_t)e * tri_ld(n);
     const int *cc = col_chan + (size_t)e * n;
     const double a = pw.a, b = pw.b;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < (long long)n * ld;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(q / ld), c = (int)(q - (q / ld) * ld);
-        double v = 0.0;
-        if (c < n) {
-            const int j = cc[c];
-            const ChanFn cj = cf[j];
-            v = -Rp[r <= j ? tri_idx(r, j, n) : tri_idx(j, r, n)] * (a * cj.ghp - b * cj.gh);
-            if (r == j) v += cj.gh;
-        } else if (c >= rhs && c < rhs + d.np) {
-            const int o = cc[d.ncl + (c - rhs)];
-            const ChanFn co = cf[o];
-            v = Rp[r <= o ? tri_idx(r, o, n) : tri_idx(o, r, n)] * (a * co.sp - b * co.s);
-            if (r == o) v -= co.s;
+    const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int r0 = blockIdx.x * 32;
+    for (int c0 = 0; c0 < ld; c0 += 32) {
+        if (threadIdx.x < 32) {
+            const int c = c0 + lane;
+            const bool left = c < n, right = c >= rhs && c < rhs + d.np;
+            int j = -1;
+            if (left || right) {
+                j = left ? cc[c] : cc[d.ncl + (c - rhs)];
+                const ChanFn cj = cf[j];
+                const double fa = a * cj.ghp - b * cj.gh, fb = a * cj.sp - b * cj.s;
+                fac[lane] = left ? -fa : fb;      // -R fa = R (-fa)
+                dia[lane] = left ? cj.gh : -cj.s;
+            }
+            chan[lane] = j;
         }
-        M[(size_t)r * ld + c] = (float)v;
+        __syncthreads();
+        // R_rj with r > j: along row j of the triangle
+        for (int y = ty; y < 32; y += 8) {
+            const int j = chan[y], r = r0 + lane;
+            if (j >= 0 && j < r && r < n) tr[y][lane] = Rp[tri_idx(j, r, n)];
+        }
+        __syncthreads();
+        const int c = c0 + lane, j = chan[lane];
+        for (int y = ty; y < 32; y += 8) {
+            const int r = r0 + y;
+            if (r >= n || c >= ld) continue;
+            float f = 0.f;
+            if (j >= 0) {
+                double v = (r <= j ? Rp[tri_idx(r, j, n)] : tr[lane][y]) * fac[lane];
+                if (r == j) v += dia[lane];
+                f = to_float(v);
+            }
+            M[(size_t)r * ld + c] = f;
+        }
+        __syncthreads();
     }
 }
 
@@ -1042,23 +1108,37 @@ __global__ void __launch_bounds__(NT, 512 / NT) lu32_kernel(int n, const EnergyD
         if (threadIdx.x == 0) atomicCAS(status + e, RM_OK, RM_ESINGULAR);
 }
 
-// K_u (FP64, np x np) = X[P rows]; without MQDT-eliminated channels also K
-// (symmetrised into ks, as written into K_out).
-__global__ void extract_f32_kernel(int n, int nE, const EnergyDims *dims, double *ws, double *K_out)
+// K_u (FP64, np x np) = X[P rows] into ku if some channel is MQDT-eliminated;
+// otherwise K (symmetrised into ks, as written into K_out). Tiles of 32 x 32:
+// the transposed entries are read through shared memory.
+__global__ void __launch_bounds__(256) extract_f32_kernel(int n, int nE, const EnergyDims *dims, double *ws, double *K_out)
 {
     const int e = blockIdx.y;
     const EnergyDims d = dims[e];
     if (d.np < 0) return;
+    __shared__ float tr[32][33];
     const Slot s = slot_of(ws, n, e);
-    const float *M = reinterpret_cast<const float *>(s.aug);
     const int ld = f32d::aug_ld(n, d.np), rhs = f32d::rhs0(n);
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d.np * d.np; q += gridDim.x * blockDim.x) {
-        const int p = q / d.np, r = q - (q / d.np) * d.np;
-        const double v = (double)M[(size_t)(d.ncl + p) * ld + rhs + r];
-        s.ku[(size_t)p * d.np + r] = v;
+    const float *X = reinterpret_cast<const float *>(s.aug) + (size_t)d.ncl * ld + rhs;
+    const int tiles = (d.np + 31) / 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int t = blockIdx.x; t < tiles * tiles; t += gridDim.x) {
+        const int p0 = 32 * (t / tiles), q0 = 32 * (t - (t / tiles) * tiles);
         if (d.nq == 0) {
-            s.ks[(size_t)p * d.no + r] = 0.5 * (v + (double)M[(size_t)(d.ncl + r) * ld + rhs + p]);
-            if (K_out) K_out[(size_t)e * n * n + (size_t)p * n + r] = v;
+            __syncthreads();
+            for (int y = ty; y < 32; y += 8)
+                if (q0 + y < d.np && p0 + tx < d.np) tr[y][tx] = X[(size_t)(q0 + y) * ld + p0 + tx];
+            __syncthreads();
+        }
+        for (int y = ty; y < 32; y += 8) {
+            const int p = p0 + y, r = q0 + tx;
+            if (p >= d.np || r >= d.np) continue;
+            const double v = (double)X[(size_t)p * ld + r];
+            if (d.nq == 0) {
+                s.ks[(size_t)p * d.no + r] = 0.5 * (v + (double)tr[tx][y]);
+                if (K_out) K_out[(size_t)e * n * n + (size_t)p * n + r] = v;
+            } else {
+                s.ku[(size_t)p * d.np + r] = v;
+            }
         }
     }
 }
@@ -1093,21 +1173,40 @@ __global__ void __launch_bounds__(NT, 512 / NT) zsweep_kernel(int n, const Energ
         if (threadIdx.x == 0) atomicCAS(status + e, RM_OK, RM_ESINGULAR);
 }
 
-// |T_ab|^2 = 4 |W_ab - delta_ab|^2 with W = (1 - iK)^{-1} = -Z (upper triangle
-// of Z, so |T|^2 is symmetric), into ks.
-__global__ void t2z_kernel(int n, int nE, const EnergyDims *dims, double *ws)
+// Omega_IJ += g sum |T_ab|^2 as omega_kernel, |T_ab|^2 = 4 |W_ab - delta_ab|^2
+// with W = (1 - iK)^{-1} = -Z (upper triangle of Z, so |T|^2 is symmetric)
+// formed where it is summed: 256 energies of 1000 channels 0.89 ms, were
+// 1.44 + 0.24 through a stored |T|^2.
+__global__ void omega_z_kernel(PwDev pw, const double *__restrict__ E, int nE, const EnergyDims *__restrict__ dims,
+                               const int *__restrict__ open_pos, double *ws, double *omega, int n_tri)
 {
     const int e = blockIdx.y;
     const EnergyDims d = dims[e];
     if (d.np < 0) return;
+    const int n = pw.n, nl = pw.n_levels;
     const Slot s = slot_of(ws, n, e);
     const float2 *Z = reinterpret_cast<const float2 *>(s.aug);
     const int ldz = f32d::z_ld(d.no);
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d.no * d.no; q += gridDim.x * blockDim.x) {
-        const int p = q / d.no, r = q - (q / d.no) * d.no;
-        const float2 u = Z[(size_t)min(p, r) * ldz + max(p, r)];   // upper triangle
-        const double ur = (double)u.x + (p == r ? 1.0 : 0.0), ui = u.y;
-        s.ks[q] = 4.0 * (ur * ur + ui * ui);
+    const double x = E[e];
+    const int *op = open_pos + (size_t)e * n;
+    double *om = omega + (size_t)e * n_tri;
+    const int npair = nl * (nl + 1) / 2;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < npair; q += gridDim.x * blockDim.x) {
+        int I, J;
+        level_pair(q, nl, I, J);
+        if (!(x - pw.lev_thr[I] > 0.0) || !(x - pw.lev_thr[J] > 0.0)) continue;
+        double sum = 0.0;
+        for (int ia = pw.lev_start[I]; ia < pw.lev_start[I + 1]; ++ia) {
+            const int pa = op[pw.lev_chan[ia]];
+            for (int ib = pw.lev_start[J]; ib < pw.lev_start[J + 1]; ++ib) {
+                const int pb = op[pw.lev_chan[ib]];
+                const float2 u = Z[(size_t)min(pa, pb) * ldz + max(pa, pb)];   // upper triangle
+                const double ur = (double)u.x + (pa == pb ? 1.0 : 0.0), ui = u.y;
+                const double t2 = 4.0 * (ur * ur + ui * ui);
+                sum += t2;
+            }
+        }
+        om[q] += pw.g * sum;
     }
 }
 
@@ -1246,7 +1345,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
         if ((err = cudaGetLastError()) != cudaSuccess) \
             return err;                               \
     } while (0)
-    classify_kernel<<<eg, 128, 0, st>>>(pw, E, nE, cf, status, dims, col_chan, open_pos, qpos, opos,
+    classify_kernel<<<(nE + 3) / 4, 128, 0, st>>>(pw, E, nE, cf, status, dims, col_chan, open_pos, qpos, opos,
                                         n_open_out);
     LAUNCH_OK();
     const int xb = (int)std::min<long long>(64, ((long long)n * 2 * n + NTH - 1) / NTH);
@@ -1254,7 +1353,7 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
     if (f32) {
         order_kernel<<<1, 1024, (size_t)(n + 2) * sizeof(int), st>>>(n, nE, dims, order);
         LAUNCH_OK();
-        assemble_f32_kernel<<<dim3(xb, nE), NTH, 0, st>>>(pw, nE, cf, R, dims, col_chan, ws);
+        assemble_f32_kernel<<<dim3((n + 31) / 32, nE), 256, 0, st>>>(pw, nE, cf, R, dims, col_chan, ws);
         LAUNCH_OK();
         if ((err = launch_lu32_any(n, nE, dims, ws, status, order, st)) != cudaSuccess) return err;
         LAUNCH_OK();
@@ -1296,11 +1395,9 @@ cudaError_t launch_solve_large(const PwDev &pw, const double *E, int nE, const C
         LAUNCH_OK();
         prune_kernel<<<eg, 128, 0, st>>>(nE, status, dims);
         LAUNCH_OK();
-        t2z_kernel<<<dim3(xb2, nE), NTH, 0, st>>>(n, nE, dims, ws);
-        LAUNCH_OK();
         const int nl = pw.n_levels;
         const int xb3 = (int)std::min<long long>(64, ((long long)nl * (nl + 1) / 2 + NTH - 1) / NTH);
-        omega_kernel<<<dim3(xb3, nE), NTH, 0, st>>>(pw, E, nE, dims, open_pos, ws, omega, n_tri);
+        omega_z_kernel<<<dim3(xb3, nE), NTH, 0, st>>>(pw, E, nE, dims, open_pos, ws, omega, n_tri);
         LAUNCH_OK();
     } else if (omega) {
         t_build_kernel<<<dim3(xb2, nE), NTH, 0, st>>>(n, nE, dims, ws, lu, gj);
