@@ -192,6 +192,12 @@ struct Lane {
     cudaEvent_t ev_solved = nullptr, ev_copied[2] = {nullptr, nullptr};
     bool copied[2] = {false, false};
     int omega_cur = 0;
+    // pieces of the last solve: the rows up to piece_end[p] are final at
+    // piece_ev[p], so that rm_collision_strengths copies them while later
+    // pieces are solved (n_pieces 0: after everything)
+    std::vector<cudaEvent_t> piece_ev;
+    std::vector<int> piece_end;
+    int n_pieces = 0;
     // workspace
     DevBuf wsE, wsCf, wsR, wsStatus, wsMq, wsDh, wsDl, wsErr, wsL, wsPart, wsDeep, wsNear, wsEhl;
     // coarse-mesh interpolation: node energies, statuses + orders, K_u, S_u, fine plan
@@ -459,6 +465,7 @@ extern "C" void rm_destroy(rm_ctx *ctx)
         if (ln->ev_solved) cudaEventDestroy(ln->ev_solved);
         for (cudaEvent_t ev : ln->ev_copied)
             if (ev) cudaEventDestroy(ev);
+        for (cudaEvent_t ev : ln->piece_ev) cudaEventDestroy(ev);
         ln->release();
         if (ln->side) cudaStreamDestroy(ln->side);
         if (ln->ev_fork) cudaEventDestroy(ln->ev_fork);
@@ -1002,11 +1009,58 @@ int tune_wave(rm_ctx *ctx, Lane *ln, PwHost &P, const double *dE, int n_E)
 
 namespace {
 
+// A solve whose Omega rows take more than this is launched in up to
+// MAX_PIECES pieces, each at least this large: the read-out of one runs beside
+// the solve of the next (20000 energies of 64 channels, 333 MB: 5.59 -> 4.31
+// ms). More pieces cost the idle SMs at each one's end more than they hide.
+constexpr size_t PIECE_BYTES = (size_t)32 << 20;
+constexpr int MAX_PIECES = 6, MAX_PIECE_EVENTS = 64;
+
+int pieces_of(int nE, int ntri)
+{
+    const size_t p = (size_t)nE * ntri * sizeof(double) / PIECE_BYTES;
+    return (int)std::min<size_t>(std::max<size_t>(p, 1), MAX_PIECES);
+}
+
+// Whether the lane's next solve may note its pieces: not while its stream is
+// being captured (an event recorded there cannot be waited for outside).
+bool may_note_pieces(Lane *ln)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ln->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
+
+// The rows before `end` are final once the work enqueued so far is done.
+cudaError_t note_piece(Lane *ln, int end)
+{
+    const size_t k = (size_t)ln->n_pieces;
+    if (k > 0 && k == MAX_PIECE_EVENTS) {   // extend the last piece
+        ln->piece_end[k - 1] = end;
+        return cudaEventRecord(ln->piece_ev[k - 1], ln->stream);
+    }
+    if (k == ln->piece_ev.size()) {
+        cudaEvent_t ev;
+        const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        ln->piece_ev.push_back(ev);
+        ln->piece_end.push_back(0);
+    }
+    ln->piece_end[k] = end;
+    const cudaError_t e = cudaEventRecord(ln->piece_ev[k], ln->stream);
+    if (e == cudaSuccess) ++ln->n_pieces;
+    return e;
+}
+
 // Registers the energy grid of the Omega accumulator (first call) or checks
 // that this call uses the registered one.
 int register_grid(rm_ctx *ctx, Lane *ln, const PwHost &P, int n_E, const double *E, bool dev_in)
 {
     const int ntri = P.n_levels * (P.n_levels + 1) / 2;
+    ln->n_pieces = 0;
     if (ln->grid_nE == 0) {
         CK(ln->omega.reserve((size_t)n_E * ntri * sizeof(double)));
         CK(cudaMemsetAsync(ln->omega.p, 0, (size_t)n_E * ntri * sizeof(double), ln->stream));
@@ -1029,8 +1083,9 @@ int register_grid(rm_ctx *ctx, Lane *ln, const PwHost &P, int n_E, const double 
 // Steps (b)-(d) for n_E device energies dE, block by block; dstatus must be
 // zeroed. omega: Omega rows of these energies (nullptr: no accumulation).
 // ku_out / ku_np (shared-memory solver, MQDT mode): K_u instead of K, T, Omega.
+// pieces: note which Omega rows are final when (note_piece).
 int solve_blocks(rm_ctx *ctx, Lane *ln, PwHost &P, const double *dE, int n_E, int mode, double *K_out, int *n_open_out,
-                 int *dstatus, double *omega, double *ku_out = nullptr, int *ku_np = nullptr)
+                 int *dstatus, double *omega, double *ku_out = nullptr, int *ku_np = nullptr, bool pieces = false)
 {
     const bool large = use_large(ctx, P);
     const int ntri = P.n_levels * (P.n_levels + 1) / 2;
@@ -1110,9 +1165,16 @@ int solve_blocks(rm_ctx *ctx, Lane *ln, PwHost &P, const double *dE, int n_E, in
             const int f32 = mode == RM_DIRECT && ctx->opts.solve_precision == RM_FP32 && !ku_out;
             double *kub = ku_out ? ku_out + (size_t)e0 * P.n * P.n : nullptr;
             int *kunb = ku_np ? ku_np + e0 : nullptr;
-            CK(launch_solve_small(d, Eb, nb, ln->wsCf.as<ChanFn>(), ln->wsR.as<double>(), sb, Kb, nob,
-                                  omb, ntri, mode == RM_MQDT, f32, deep, 0, ln->stream, kub, kunb));
-            ++ctx->launches;
+            const int np = pieces && !split ? pieces_of(nb, ntri) : 1;
+            for (int p = 0; p < np; ++p) {
+                const size_t a = (size_t)nb * p / np, b = (size_t)nb * (p + 1) / np;
+                CK(launch_solve_small(d, Eb + a, (int)(b - a), ln->wsCf.as<ChanFn>() + a * P.n,
+                                      ln->wsR.as<double>() + a * tri_ld(P.n), sb + a, Kb ? Kb + a * P.n * P.n : nullptr,
+                                      nob ? nob + a : nullptr, omb ? omb + a * ntri : nullptr, ntri, mode == RM_MQDT, f32,
+                                      deep, 0, ln->stream, kub ? kub + a * P.n * P.n : nullptr, kunb ? kunb + a : nullptr));
+                ++ctx->launches;
+                if (p + 1 < np) CK(note_piece(ln, e0 + (int)b));
+            }
             if (split) {
                 CK(cudaStreamWaitEvent(ln->stream, ln->ev_join, 0));
                 CK(launch_solve_small(d, Eb, nb, ln->wsCf.as<ChanFn>(), ln->wsR.as<double>(), sb, Kb, nob,
@@ -1121,6 +1183,8 @@ int solve_blocks(rm_ctx *ctx, Lane *ln, PwHost &P, const double *dE, int n_E, in
             }
         }
         CK(prof_end(ctx, RM_PH_SOLVE, ln->stream));
+        // a single piece is left to the plain read-out
+        if (pieces && (e0 + nb < n_E || ln->n_pieces > 0)) CK(note_piece(ln, e0 + nb));
     }
     return RM_SUCCESS;
 }
@@ -1172,8 +1236,12 @@ int solve_on_lane(rm_ctx *ctx, int lane, int pw, int n_E, const double *E, int m
         dstatus = ln->wsStatus.as<int>();
     }
     CK(cudaMemsetAsync(dstatus, 0, (size_t)n_E * sizeof(int), ln->stream));
-    rc = solve_blocks(ctx, ln, P, dE, n_E, mode, K_out, n_open_out, dstatus, ln->omega.as<double>());
-    if (rc) return rc;
+    rc = solve_blocks(ctx, ln, P, dE, n_E, mode, K_out, n_open_out, dstatus, ln->omega.as<double>(), nullptr, nullptr,
+                      may_note_pieces(ln));
+    if (rc) {
+        ln->n_pieces = 0;
+        return rc;
+    }
     CK(cudaEventRecord(ln->ev_done, ln->stream));
     return RM_SUCCESS;
 }
@@ -1282,14 +1350,31 @@ extern "C" int rm_solve_energies_qdt(rm_ctx *ctx, int pw, int n_E, const double 
     }
     CK(cudaMemsetAsync(dstatus, 0, (size_t)n_E * sizeof(int), ln->stream));
     const int ntri = P.n_levels * (P.n_levels + 1) / 2;
-    CK(launch_qdt_fine(iqdt, P.dev_match(), dE, n_E, make_opts(ctx->opts), ln->wsQf.as<QdtFine>(),
-                       ln->wsQk.as<double>(), ln->wsQs.as<double2>(), ln->wsQst.as<int>(), dstatus,
-                       n_open_out, ln->omega.as<double>(), ntri, ln->stream));
+    const int np = may_note_pieces(ln) ? pieces_of(n_E, ntri) : 1;
+    for (int p = 0; p < np; ++p) {
+        const size_t a = (size_t)n_E * p / np, b = (size_t)n_E * (p + 1) / np;
+        CK(launch_qdt_fine(iqdt, P.dev_match(), dE + a, (int)(b - a), make_opts(ctx->opts), ln->wsQf.as<QdtFine>() + a,
+                           ln->wsQk.as<double>(), ln->wsQs.as<double2>(), ln->wsQst.as<int>(), dstatus + a,
+                           n_open_out ? n_open_out + a : nullptr, ln->omega.as<double>() + a * ntri, ntri, ln->stream));
+        if (np > 1) CK(note_piece(ln, (int)b));
+        if (p > 0) ctx->launches++;
+    }
     ctx->launches++;
     return RM_SUCCESS;
 }
 
 namespace {
+
+// The lane's copy stream and its events (created on first use).
+int copy_stream(rm_ctx *ctx, Lane *ln)
+{
+    if (ln->copy) return RM_SUCCESS;
+    if (!ln->ev_solved) CK(cudaEventCreateWithFlags(&ln->ev_solved, cudaEventDisableTiming));
+    for (cudaEvent_t &ev : ln->ev_copied)
+        if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    CK(cudaStreamCreateWithFlags(&ln->copy, cudaStreamNonBlocking));
+    return RM_SUCCESS;
+}
 
 int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset)
 {
@@ -1299,12 +1384,30 @@ int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset
         return fail(ctx, RM_EINVAL, "no energy grid registered yet");
     }
     const size_t bytes = (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double);
-    if (omega_out)
+    if (omega_out && ln->n_pieces > 1 && ln->piece_end[ln->n_pieces - 1] == ln->grid_nE) {
+        int rc = copy_stream(ctx, ln);
+        if (rc) return rc;
+        cudaError_t err = cudaSuccess;
+        int e0 = 0;
+        for (int p = 0; p < ln->n_pieces && err == cudaSuccess; ++p) {
+            const size_t off = (size_t)e0 * ln->grid_ntri, cnt = (size_t)(ln->piece_end[p] - e0) * ln->grid_ntri;
+            err = cudaStreamWaitEvent(ln->copy, ln->piece_ev[p], 0);
+            if (err == cudaSuccess)
+                err = cudaMemcpyAsync(omega_out + off, ln->omega.as<double>() + off, cnt * sizeof(double),
+                                      cudaMemcpyDeviceToHost, ln->copy);
+            e0 = ln->piece_end[p];
+        }
+        const cudaError_t err2 = cudaStreamSynchronize(ln->copy);   // nothing writes omega_out after the return
+        CK(err);
+        CK(err2);
+    } else if (omega_out) {
         CK(cudaMemcpyAsync(omega_out, ln->omega.p, bytes, cudaMemcpyDeviceToHost, ln->stream));
+    }
     CK(cudaStreamSynchronize(ln->stream));
     int rc = check_device_flag(ctx, ln);
     if (rc) return rc;
     if (reset) {
+        ln->n_pieces = 0;
         ln->grid_nE = ln->grid_nlev = ln->grid_ntri = 0;
         ln->grid_host.clear();
     }
@@ -1366,12 +1469,9 @@ extern "C" int rm_collision_strengths_async(rm_ctx *ctx, double *omega_out, int 
     if (!omega_out) return fail(ctx, RM_EINVAL, "omega_out is NULL");
     if (ln->grid_nE == 0) return fail(ctx, RM_EINVAL, "no energy grid registered yet");
     CK(cudaSetDevice(ctx->opts.device));
-    if (!ln->copy) {
-        CK(cudaStreamCreateWithFlags(&ln->copy, cudaStreamNonBlocking));
-        CK(cudaEventCreateWithFlags(&ln->ev_solved, cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&ln->ev_copied[0], cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&ln->ev_copied[1], cudaEventDisableTiming));
-    }
+    const int crc = copy_stream(ctx, ln);
+    if (crc) return crc;
+    ln->n_pieces = 0;
     const size_t bytes = (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double);
     const int cur = ln->omega_cur;
     CK(cudaEventRecord(ln->ev_solved, ln->stream));
@@ -1400,6 +1500,7 @@ extern "C" int rm_reset_omega(rm_ctx *ctx)
     Lane *ln = &ctx->lanes[0];
     if (ln->grid_nE == 0) return fail(ctx, RM_EINVAL, "no energy grid registered yet");
     CK(cudaSetDevice(ctx->opts.device));
+    ln->n_pieces = 0;
     CK(cudaMemsetAsync(ln->omega.p, 0, (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double),
                        ln->stream));
     return RM_SUCCESS;
@@ -1621,6 +1722,7 @@ extern "C" int rm_solve_batch(rm_ctx *ctx, int n_pw, const int *pws, int n_E, co
         if (rc) return rc;
     }
     CK(cudaSetDevice(ctx->opts.device));
+    for (Lane &l : ctx->lanes) l.n_pieces = 0;
     Lane *l0 = &ctx->lanes[0];
     PwHost &P0 = ctx->pw[pws[0]];
     const bool dev_in = is_device_ptr(E);
