@@ -94,6 +94,21 @@ __device__ __forceinline__ PeItem pe_decode(const PeGeom &g, long long item)
     return it;
 }
 
+// Columns [lo, hi) of tile (ib, jb) that hold some i <= j < n, in halves of 128:
+// the left half lies below the diagonal when the rows start at its end, the
+// right half may lie past the last channel. 20 tiles of 1000 channels are 18,
+// 5 of 331 are 3, 2 of 231 are 1.5: 256 energies of 1000 channels 15.9 ms, were
+// 16.6, 512 of 331 2.52, were 2.69 (a half tile takes more than half the time:
+// its scaled operand is converted all the same).
+struct PeCols {
+    int lo, hi;
+};
+__device__ __forceinline__ PeCols pe_cols(const PeGeom &g, const PeItem &it)
+{
+    return {it.ib * PE_BM >= it.jb * PE_BN + PE_BN / 2 ? PE_BN / 2 : 0,
+            g.n - it.jb * PE_BN <= PE_BN / 2 ? PE_BN / 2 : PE_BN};
+}
+
 // Lane 0 waits, the warp follows its verdict (keeps .sync.aligned
 // instructions and __syncwarp convergent if a wait gives up).
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int *err, int lane)
@@ -209,25 +224,26 @@ __global__ void __launch_bounds__(PE_THREADS, 1)
     } else if (warp == 1) {
         if (lane == 0) {
             // ---- MMA issuer ----
-            const uint32_t id = idesc<KIND, PE_BM, PE_BN>();
             int bs = 0, as = 0;
             uint32_t bph = 0, aph = 0, eph = 0;
             bool ok = true;
             for (long long item = blockIdx.x; ok && item < g.n_items; item += gridDim.x) {
                 const PeItem it = pe_decode(g, item);
+                const PeCols co = pe_cols(g, it);
+                const uint32_t id = co.hi - co.lo == PE_BN ? idesc<KIND, PE_BM, PE_BN>() : idesc<KIND, PE_BM, PE_BN / 2>();
                 if (!mbar_wait(acce, eph ^ 1u, err_flag)) { ok = false; break; }
                 tc_fence_after();
                 for (int c = it.c0; ok && c < it.c1; ++c) {
                     if (!mbar_wait(&bfull[bs], bph, err_flag)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t b = smem_u32(bring + bs * PE_B_STAGE);
+                    const uint32_t b = smem_u32(bring + bs * PE_B_STAGE) + (uint32_t)(co.lo * TC_ROW_BYTES);
                     const uint64_t bh = sdesc_sw128(b), bl = sdesc_sw128(b + PE_B_TILE);
                     for (int j = 0; j < it.ng; ++j) {
                         if (!mbar_wait(&afull[as], aph, err_flag)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t a = smem_u32(aring + as * PE_A_SLOT);
                         const uint64_t ah = sdesc_sw128(a), al = sdesc_sw128(a + PE_A_TILE);
-                        const uint32_t d = tmem + (uint32_t)(j * PE_BN);
+                        const uint32_t d = tmem + (uint32_t)(j * PE_BN + co.lo);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) {
                             const uint64_t o = (uint64_t)(ks * 32) >> 4;   // 32 bytes of K per MMA
@@ -257,12 +273,13 @@ __global__ void __launch_bounds__(PE_THREADS, 1)
         uint32_t fph = 0;
         for (long long item = blockIdx.x; item < g.n_items; item += gridDim.x) {
             const PeItem it = pe_decode(g, item);
+            const PeCols co = pe_cols(g, it);
             if (!warp_wait(accf, fph, err_flag, lane)) break;
             tc_fence_after();
             for (int j = 0; j < it.ng; ++j) {
                 float *row = part + ((((size_t)it.seg * g.nE + it.e0 + j) * g.n_tiles + it.t) * PE_BM + il) *
                                         PE_BN;
-                for (int c0 = 0; c0 < PE_BN; c0 += 32) {
+                for (int c0 = co.lo; c0 < co.hi; c0 += 32) {
                     uint32_t r[32];
                     tmem_ld32(tmem + (uint32_t)(j * PE_BN + c0) + ((uint32_t)(quad * 32) << 16), r);
 #pragma unroll

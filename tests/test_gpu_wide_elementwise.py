@@ -61,3 +61,22 @@ def test_omega_against_fp64_solver(n, per, mode):
     assert np.array_equal(ref == 0.0, om == 0.0)
     off = np.linalg.norm(om - ref, axis=1) / np.linalg.norm(ref, axis=1)
     assert np.median(off) <= n * 2.0 ** -18, off
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 255, 256, 257, 383, 385])
+@pytest.mark.parametrize("prec", [rmgb.RM_BF16X3, rmgb.RM_FP32])
+def test_formation_tiles(n, prec):
+    """Per-energy formation where its 128 x 256 tiles are computed by halves: every entry within the mixed
+    formation's bound (a half left out is an error of order one)."""
+    pw = synth.random_pw(n, n, 2 * n + 70, z=2.0, a=15.0, sigma=0.05)
+    E = np.array([0.3, 0.9, 2.2])
+    with rmgb.Context(precision=prec, formulation=rmgb.RM_FORM_ENERGY) as ctx:
+        ctx.load_pw(0, pw)
+        R = torch.full((3, n, n), float("nan"), dtype=torch.float64, device="cuda")
+        ctx.form_r(0, torch.tensor(E, device="cuda"), R)
+        ctx.sync()
+        R = R.cpu().numpy()
+    for e in range(3):
+        d = 1.0 / (pw["E_k"] - E[e])
+        ref, S = (pw["W"] * d) @ pw["W"].T / 30.0, (abs(pw["W"]) * abs(d)) @ abs(pw["W"]).T / 30.0
+        assert np.all(np.abs(R[e] - ref) <= 1e-4 * S)
