@@ -676,40 +676,45 @@ __device__ void chanfn_pair(const PwDev &pw, const double *__restrict__ E, int n
 }
 
 
-// ---- four lanes per pair -----------------------------------------------------
+// ---- several lanes per pair ----------------------------------------------------
 //
 // Without channel tables (z = 0, FP64 contexts, rm_k_matrices_noalloc) every
 // pair runs its continued fractions, and a launch lasts as long as the deepest
 // one: a warp's FP64 instruction holds its quarter of the SM's FP64 unit for 64
 // clocks, however few of its lanes are at work, and a step of CF2 took 24 of
-// them. Here four lanes share a pair: the recurrences' components (A and B,
-// real and imaginary) go one to a lane, the coefficients of eight steps two to
-// a lane, so a step of CF2 takes 9 (forwards) or 4 (backwards) instructions.
-// Each operation is the one of cf1_lentz, cf2_open_l0, cf2_closed,
+// them. Here W = 4 or 8 lanes share a pair: the recurrences' components (A and
+// B, real and imaginary) go one to a lane, the coefficients of eight steps 8 / W
+// to a lane, so a step of CF2 takes 9 (W = 8: 6) instructions forwards and 4 (3)
+// backwards. Each operation is the one of cf1_lentz, cf2_open_l0, cf2_closed,
 // open_channel and closed_channel above, on the same operands: the results are
-// the same to the bit. 16 energies of 4 channels: 134 us, was 270; 2000 of 4
-// channels 450 us, was 906; 4000 of 64 channels 1.72 ms, was 2.07.
-constexpr int X4_BS = 128;                // threads per block: 32 pairs
-constexpr int X4_PAIRS = X4_BS / 4;
+// the same to the bit. One thread, four lanes, eight lanes: 16 energies of 4
+// channels 270, 134, 106 us; 2000 of 4 906, 450, 395; 304 of 32 830, 432, 336;
+// 200 of 132 654, 500, 516; 1777 of 41 (z = 0) 2211, 252, 385; 4000 of 64 2.07,
+// 1.72, 2.03 ms. Up to XN_W8_PAIRS pairs leave the SMs room for eight lanes.
+constexpr int XN_BS = 128;                // threads per block
+constexpr long long XN_W8_PAIRS = 16384;
 // z = 0: from this k a (kappa a) on, the fractions whose first numerator is
 // zero are not run for their tail, which converges there in well under
 // CF_MAXIT steps; nearer a threshold they are run as ever, and a tail that
 // does not converge fails its energy as ever.
-constexpr double X4_Z0_MIN = 0.02;
+constexpr double XN_Z0_MIN = 0.02;
 
-// The four lanes of a pair: c = 0..3.
-struct Quad {
+// The W lanes of a pair: c = 0 .. W - 1. Lane c has component c % 4 (A real, A
+// imaginary, B real, B imaginary; real fractions: A on even, B on odd lanes).
+template <int W> struct Lanes {
     int c;
     unsigned mask;
-    __device__ __forceinline__ Quad() : c(threadIdx.x & 3), mask(0xfu << (threadIdx.x & 28)) {}
-    __device__ __forceinline__ double get(double v, int src) const { return __shfl_sync(mask, v, src, 4); }
-    __device__ __forceinline__ double swap(double v) const { return __shfl_xor_sync(mask, v, 1, 4); }
-    // pow2_rescale of the largest magnitude among the lanes' v (and w)
+    __device__ __forceinline__ Lanes() : c(threadIdx.x & (W - 1)),
+                                         mask((W == 8 ? 0xffu : 0xfu) << (threadIdx.x & 31 & ~(W - 1))) {}
+    __device__ __forceinline__ double get(double v, int src) const { return __shfl_sync(mask, v, src, W); }
+    // coefficient of step k of a block of eight, from the lane that formed it
+    __device__ __forceinline__ double coef(const double (&v)[8 / W], int k) const { return get(v[k / W], k % W); }
+    // pow2_rescale of the largest magnitude among the lanes' v and w
     __device__ __forceinline__ double rescale(double v, double w) const
     {
         int ex = max((__double2hiint(v) >> 20) & 0x7ff, (__double2hiint(w) >> 20) & 0x7ff);
-        ex = max(ex, __shfl_xor_sync(mask, ex, 1, 4));
-        ex = max(ex, __shfl_xor_sync(mask, ex, 2, 4));
+        ex = max(ex, __shfl_xor_sync(mask, ex, 1, W));
+        ex = max(ex, __shfl_xor_sync(mask, ex, 2, W));
         int se = 2046 - ex;
         se = se < 1 ? 1 : (se > 2046 ? 2046 : se);
         return __hiloint2double(se << 20, 0);
@@ -721,100 +726,148 @@ __device__ __forceinline__ double neg_if(double v, bool neg)
     return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
 }
 
-__device__ Cf1 cf1_lentz_x4(const Quad &g, int l, double eta, double rho)
-{
-    const double irho = 1.0 / rho;
-    const double L1 = l + 1.0;
-    double er_last = eta / L1;
-    double S_last = L1 * irho + er_last;
-    const bool isA = !(g.c & 1);
-    double own1 = isA ? S_last : 1.0, own2 = isA ? 1.0 : 0.0;   // A or B of n - 1, n - 2
-    for (int n0 = 1; n0 + CF_CHECK - 1 < CF_MAXIT; n0 += CF_CHECK) {
-        // steps n0 + c and n0 + 4 + c: a_n, b_n
-        double an[2], bn[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const double Ln1 = l + (n0 + 4 * h + g.c) + 1.0;
-            const double er1 = eta * rcp_nr(Ln1);
-            const double Snext = Ln1 * irho + er1;
-            const double er_up = __shfl_up_sync(g.mask, er1, 1, 4), S_up = __shfl_up_sync(g.mask, Snext, 1, 4);
-            const double er = g.c ? er_up : er_last, S = g.c ? S_up : S_last;
-            an[h] = -fma(er, er, 1.0);
-            bn[h] = S + Snext;
-            er_last = g.get(er1, 3);
-            S_last = g.get(Snext, 3);
-        }
-#pragma unroll
-        for (int k = 0; k < CF_CHECK; ++k) {
-            const double a = g.get(an[k >> 2], k & 3), b = g.get(bn[k >> 2], k & 3);
-            const double v = fma(b, own1, a * own2);
+// The recurrence X_n = b_n X_{n-1} + a_n X_{n-2} of A and B, real. W = 8: lanes
+// 0..3 form fma(b_n, X_{n-1}, u_n) and lanes 4..7 u_{n+1} = a_{n+1} X_{n-1}
+// (exactly, as fma(a, X, -0)) in one instruction.
+template <int W> struct RealPair {
+    double own1, own2, u;   // X_{n-1}, X_{n-2} of this lane's A or B; a_n X_{n-2}
+    __device__ __forceinline__ void step(const Lanes<W> &g, double b, double a_next)
+    {
+        if constexpr (W == 8) {
+            const bool T = g.c >= 4;
+            const double y = fma(T ? a_next : b, own1, T ? -0.0 : u);
             own2 = own1;
-            own1 = v;
+            own1 = g.get(y, g.c & 1);
+            u = g.get(y, 4 + (g.c & 1));
+        } else {
+            const double y = fma(b, own1, u);
+            u = a_next * own1;
+            own2 = own1;
+            own1 = y;
         }
+    }
+    // rescales, then A_n / B_n and A_{n-1} / B_{n-1}; the sign of B_n
+    __device__ __forceinline__ bool ratios(const Lanes<W> &g, double *f, double *fp)
+    {
         const double sc = g.rescale(own1, own2);
         own1 *= sc;
         own2 *= sc;
+        u *= sc;
         const double A1 = g.get(own1, 0), B1 = g.get(own1, 1), A2 = g.get(own2, 0), B2 = g.get(own2, 1);
-        const double q = (g.c < 2 ? A1 : A2) / (g.c < 2 ? B1 : B2);
-        const double f = g.get(q, 0), fp = g.get(q, 2);
-        if (fabs(f - fp) < CF_TOL * fabs(fp)) return {f, B1 < 0.0 ? -1 : 1, 1, n0 + CF_CHECK - 1};
+        const bool first = g.c < W / 2;
+        const double q = (first ? A1 : A2) / (first ? B1 : B2);
+        *f = g.get(q, 0);
+        *fp = g.get(q, W / 2);
+        return B1 < 0.0;
+    }
+};
+
+template <int W> __device__ Cf1 cf1_lentz_xn(const Lanes<W> &g, int l, double eta, double rho)
+{
+    constexpr int H = 8 / W;
+    const double irho = 1.0 / rho;
+    const double L1 = l + 1.0;
+    const double er0 = eta / L1;
+    double S_last = L1 * irho + er0;   // S_{n0 - 1}
+    const bool isA = !(g.c & 1);
+    RealPair<W> x;
+    x.own1 = isA ? S_last : 1.0;
+    x.own2 = isA ? 1.0 : 0.0;
+    x.u = -fma(er0, er0, 1.0) * x.own2;
+    for (int n0 = 1; n0 + CF_CHECK - 1 < CF_MAXIT; n0 += CF_CHECK) {
+        double a1[H], bn[H];   // a_{n+1} = -(1 + er_n^2), b_n = S_{n-1} + S_n
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const double Ln1 = l + (n0 + W * h + g.c) + 1.0;
+            const double er = eta * rcp_nr(Ln1);
+            const double S = Ln1 * irho + er;
+            const double up = __shfl_up_sync(g.mask, S, 1, W);
+            a1[h] = -fma(er, er, 1.0);
+            bn[h] = (g.c ? up : S_last) + S;
+            S_last = g.get(S, W - 1);
+        }
+#pragma unroll
+        for (int k = 0; k < CF_CHECK; ++k) x.step(g, g.coef(bn, k), g.coef(a1, k));
+        double f, fp;
+        const bool neg = x.ratios(g, &f, &fp);
+        if (fabs(f - fp) < CF_TOL * fabs(fp)) return {f, neg ? -1 : 1, 1, n0 + CF_CHECK - 1};
     }
     return {0.0, 1, 0, CF_MAXIT};
 }
 
-__device__ int cf2_open_l0_x4(const Quad &g, double eta, double rho, double *p, double *q)
+template <int W> __device__ int cf2_open_l0_xn(const Lanes<W> &g, double eta, double rho, double *p, double *q)
 {
+    constexpr int H = 8 / W;
     // z = 0: a_1 = 0, so K = 0 whatever its tail, and H+ = exp(i rho)
-    if (eta == 0.0 && rho >= X4_Z0_MIN) {
+    if (eta == 0.0 && rho >= XN_Z0_MIN) {
         *p = 0.0;
         *q = 1.0;
         return 1;
     }
     const double br = 2.0 * (rho - eta);
-    const bool im = g.c & 1, hi2 = g.c >> 1;
-    // lanes: A real, A imaginary, B real, B imaginary of m - 1 (1) and m - 2 (2)
-    double own1 = hi2 ? (im ? 0.0 : 1.0) : (im ? 2.0 : br), own2 = hi2 ? 0.0 : (im ? 0.0 : 1.0);
-    double oth1 = g.swap(own1), oth2 = g.swap(own2);
-    double fr = br, fi = 2.0;
-    int n = 0;
-    bool conv = false;
-    auto coef = [&](int m_, double &ar, double &ai, double &bi) {
+    const bool im = g.c & 1, B = g.c & 2, T = g.c >= 4;
+    const int comp = g.c & 3;
+    auto a_of = [&](int m_, double &ar, double &ai) {
         const double m = m_;
         ar = m * (m - 1.0) - eta * eta;
         ai = eta * (2.0 * m - 1.0);
-        bi = 2.0 * m;
     };
+    // this lane's component of m - 1 (own1; oth1: its partner's) and m - 2
+    // (own2), and of the product a_m X_{m-2} (u)
+    double own1 = B ? (im ? 0.0 : 1.0) : (im ? 2.0 : br), own2 = B ? 0.0 : (im ? 0.0 : 1.0);
+    double oth1 = g.get(own1, g.c ^ 1), u;
+    {
+        double ar, ai;
+        a_of(2, ar, ai);
+        u = fma(ar, own2, neg_if(ai, !im) * g.get(own2, g.c ^ 1));
+    }
+    double fr = br, fi = 2.0;
+    int n = 0;
+    bool conv = false;
     for (int n0 = 1; n0 + CF_CHECK - 1 < CF_MAXIT; n0 += CF_CHECK) {
-        double car[2], cai[2], cbi[2];
+        double car[H], cai[H], cbi[H];   // a of step n + 1, b of step n
 #pragma unroll
-        for (int h = 0; h < 2; ++h) coef(n0 + 4 * h + g.c, car[h], cai[h], cbi[h]);
+        for (int h = 0; h < H; ++h) {
+            const int m = n0 + W * h + g.c;
+            a_of(m + 1, car[h], cai[h]);
+            cbi[h] = 2.0 * (double)m;
+        }
 #pragma unroll
         for (int k = 0; k < CF_CHECK; ++k) {
-            const double ar = g.get(car[k >> 2], k & 3);
-            const double ai = neg_if(g.get(cai[k >> 2], k & 3), !im), bi = neg_if(g.get(cbi[k >> 2], k & 3), !im);
+            const double ar = g.coef(car, k), ai = neg_if(g.coef(cai, k), !im), bi = neg_if(g.coef(cbi, k), !im);
             if (k > 0 || n0 > 1) {   // the first step is m = 2
-                const double t = fma(ar, own2, ai * oth2);
-                const double v = fma(br, own1, fma(bi, oth1, t));
-                own2 = own1;
-                oth2 = oth1;
-                own1 = v;
-                oth1 = g.swap(v);
+                if constexpr (W == 8) {
+                    const double t = fma(T ? ai : bi, oth1, T ? -0.0 : u);
+                    const double y = fma(T ? ar : br, own1, t);
+                    own2 = own1;
+                    own1 = g.get(y, comp);
+                    oth1 = g.get(y, comp ^ 1);
+                    u = g.get(y, 4 + comp);
+                } else {
+                    const double y = fma(br, own1, fma(bi, oth1, u));
+                    u = fma(ar, own1, ai * oth1);
+                    own2 = own1;
+                    own1 = y;
+                    oth1 = g.get(y, g.c ^ 1);
+                }
             }
         }
         const double sc = g.rescale(own1, own2);
         own1 *= sc;
         own2 *= sc;
         oth1 *= sc;
-        oth2 *= sc;
+        u *= sc;
+        // the convergent of n on the first half of the lanes, of n - 1 on the other
+        const bool first = g.c < W / 2;
         const double x0 = g.get(own1, 0), x1 = g.get(own1, 1), x2 = g.get(own1, 2), x3 = g.get(own1, 3);
         const double y0 = g.get(own2, 0), y1 = g.get(own2, 1), y2 = g.get(own2, 2), y3 = g.get(own2, 3);
-        const double A1r = hi2 ? y0 : x0, A1i = hi2 ? y1 : x1, B1r = hi2 ? y2 : x2, B1i = hi2 ? y3 : x3;
+        const double A1r = first ? x0 : y0, A1i = first ? x1 : y1, B1r = first ? x2 : y2, B1i = first ? x3 : y3;
         const double d1 = 1.0 / (B1r * B1r + B1i * B1i);
         const double cr = (A1r * B1r + A1i * B1i) * d1;
         const double ci = (A1i * B1r - A1r * B1i) * d1;
         fr = g.get(cr, 0);
         fi = g.get(ci, 0);
-        const double gr = g.get(cr, 2), gi = g.get(ci, 2);
+        const double gr = g.get(cr, W / 2), gi = g.get(ci, W / 2);
         if (fabs(fr - gr) + fabs(fi - gi) < CF_TOL * (fabs(gr) + fabs(gi))) {
             conv = true;
             n = n0 + CF_CHECK - 1;
@@ -830,25 +883,27 @@ __device__ int cf2_open_l0_x4(const Quad &g, double eta, double rho, double *p, 
         *q = (1.0 - eta / rho) + ((ar * fr + ai * fi) * dm) / rho;
         return 1;
     }
-    // backwards from N: lanes p real, p imaginary, q real, q imaginary
+    // backwards from N: components p real, p imaginary, q real, q imaginary;
+    // p <- a_m q (the product exactly as a_i q_i + -0), q <- p + b_m q
     const int N = 2 * n + 20;
-    double v = (g.c == 2) ? 1.0 : 0.0;
-    const double w2 = br;
+    double v = comp == 2 ? 1.0 : 0.0;
     for (int j = N / CF_CHECK; j >= 0; --j) {
-        double car[2], cai[2], cbi[2];
+        double car[H], cai[H], cbi[H];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) coef(CF_CHECK * j + 4 * h + g.c, car[h], cai[h], cbi[h]);
+        for (int h = 0; h < H; ++h) {
+            const int m = CF_CHECK * j + W * h + g.c;
+            a_of(m, car[h], cai[h]);
+            cbi[h] = 2.0 * (double)m;
+        }
 #pragma unroll
         for (int k = CF_CHECK - 1; k >= 0; --k) {
-            const double ar = g.get(car[k >> 2], k & 3);
-            const double ai = g.get(cai[k >> 2], k & 3), bi = g.get(cbi[k >> 2], k & 3);
+            const double ar = g.coef(car, k), ai = g.coef(cai, k), bi = g.coef(cbi, k);
             const int m_ = CF_CHECK * j + k;
             if (m_ > N || m_ < 1) continue;
             const double qown = g.get(v, 2 + (g.c & 1)), qoth = g.get(v, 2 + ((g.c & 1) ^ 1));
             const double pown = g.get(v, g.c & 1);
-            // p <- a_m q (the product exactly as a_i q_i + -0), q <- p + b_m q
-            const double t = fma(neg_if(hi2 ? bi : ai, !im), qoth, hi2 ? pown : -0.0);
-            v = fma(hi2 ? w2 : ar, qown, t);
+            const double t = fma(neg_if(B ? bi : ai, !im), qoth, B ? pown : -0.0);
+            v = fma(B ? br : ar, qown, t);
         }
         if (j > 0) v *= g.rescale(v, v);
     }
@@ -863,45 +918,39 @@ __device__ int cf2_open_l0_x4(const Quad &g, double eta, double rho, double *p, 
 // MQDT: the one-thread kernels round kappa a before subtracting nu in the
 // quantum-defect mode (the product is compared with its cap as well) and
 // contract the two in the direct mode; so does this.
-template <bool MQDT>
-__device__ int cf2_closed_x4(const Quad &g, int L0, double nu, double kap, double a, double *y)
+template <bool MQDT, int W>
+__device__ int cf2_closed_xn(const Lanes<W> &g, int L0, double nu, double kap, double a, double *y)
 {
+    constexpr int H = 8 / W;
     const double base = MQDT ? __dsub_rn(__dmul_rn(kap, a), nu) : fma(kap, a, -nu);
     auto an = [&](int m) { return (L0 + m - nu) * (m - 1.0 - L0 - nu); };
     // z = 0 at L0 = 0: a_1 = 0, so the fraction is 0 whatever its tail
-    if (an(1) == 0.0 && nu == 0.0 && kap * a >= X4_Z0_MIN) {
+    if (an(1) == 0.0 && nu == 0.0 && kap * a >= XN_Z0_MIN) {
         *y = -kap;
         return 1;
     }
     const bool isA = !(g.c & 1);
-    double own1 = isA ? 2.0 * (base + 1.0) : 1.0, own2 = isA ? 1.0 : 0.0;
-    double f = 0.0;
+    RealPair<W> x;
+    x.own1 = isA ? 2.0 * (base + 1.0) : 1.0;
+    x.own2 = isA ? 1.0 : 0.0;
+    x.u = -an(2) * x.own2;
+    double f = 0.0, fp;
     int n = 0;
     bool conv = false;
     for (int n0 = 1; n0 + CF_CHECK - 1 < CF_MAXIT; n0 += CF_CHECK) {
-        double num[2], den[2];
+        double num[H], den[H];   // numerator of step m + 1, denominator of step m
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int m = n0 + 4 * h + g.c;
-            num[h] = -an(m);
+        for (int h = 0; h < H; ++h) {
+            const int m = n0 + W * h + g.c;
+            num[h] = -an(m + 1);
             den[h] = 2.0 * (base + m);
         }
 #pragma unroll
         for (int k = 0; k < CF_CHECK; ++k) {
-            const double nm = g.get(num[k >> 2], k & 3), dn = g.get(den[k >> 2], k & 3);
-            if (k > 0 || n0 > 1) {   // the first step is m = 2
-                const double v = fma(dn, own1, nm * own2);
-                own2 = own1;
-                own1 = v;
-            }
+            const double dn = g.coef(den, k), nm = g.coef(num, k);
+            if (k > 0 || n0 > 1) x.step(g, dn, nm);   // the first step is m = 2
         }
-        const double sc = g.rescale(own1, own2);
-        own1 *= sc;
-        own2 *= sc;
-        const double A1 = g.get(own1, 0), B1 = g.get(own1, 1), A2 = g.get(own2, 0), B2 = g.get(own2, 1);
-        const double q = (g.c < 2 ? A1 : A2) / (g.c < 2 ? B1 : B2);
-        f = g.get(q, 0);
-        const double fp = g.get(q, 2);
+        x.ratios(g, &f, &fp);
         if (fabs(f - fp) < CF_TOL * fabs(fp)) {
             conv = true;
             n = n0 + CF_CHECK - 1;
@@ -917,16 +966,16 @@ __device__ int cf2_closed_x4(const Quad &g, int L0, double nu, double kap, doubl
     const int N = 2 * n + 20;
     double v = isA ? 0.0 : 1.0;
     for (int j = N / CF_CHECK; j >= 0; --j) {
-        double num[2], den[2];
+        double num[H], den[H];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int m = CF_CHECK * j + 4 * h + g.c;
+        for (int h = 0; h < H; ++h) {
+            const int m = CF_CHECK * j + W * h + g.c;
             num[h] = -an(m);
             den[h] = 2.0 * (base + m);
         }
 #pragma unroll
         for (int k = CF_CHECK - 1; k >= 0; --k) {
-            const double nm = g.get(num[k >> 2], k & 3), dn = g.get(den[k >> 2], k & 3);
+            const double nm = g.coef(num, k), dn = g.coef(den, k);
             const int m = CF_CHECK * j + k;
             if (m > N || m < 2) continue;
             const double qq = g.get(v, 1), pp = g.get(v, 0);
@@ -939,33 +988,32 @@ __device__ int cf2_closed_x4(const Quad &g, int L0, double nu, double kap, doubl
     return 1;
 }
 
-// S_L = L / rho + eta / L and R_L = sqrt(1 + eta^2 / L^2) of L = 4 j + 1 + c.
+// S_L = L / rho + eta / L and R_L = sqrt(1 + eta^2 / L^2).
 __device__ __forceinline__ void coulomb_sr(int L, double eta, double rho, double *S, double *R)
 {
     *S = L / rho + eta / L;
     *R = sqrt(1.0 + (eta / L) * (eta / L));
 }
 
-__device__ int open_channel_x4(const Quad &g, int l, double eps, double z, double a, double *s, double *sp, double *c,
+template <int W>
+__device__ int open_channel_xn(const Lanes<W> &g, int l, double eps, double z, double a, double *s, double *sp, double *c,
                                double *cp)
 {
     const double k = sqrt(eps);
     const double eta = -z / k;
     const double rho = k * a;
-    const Cf1 c1 = cf1_lentz_x4(g, l, eta, rho);
+    const Cf1 c1 = cf1_lentz_xn(g, l, eta, rho);
     double p, q;
-    const int ok2 = cf2_open_l0_x4(g, eta, rho, &p, &q);
+    const int ok2 = cf2_open_l0_xn(g, eta, rho, &p, &q);
     if (!c1.ok || !ok2) return 0;
     // F_l, F_l' up to a common scale, carried down to l = 0
     const double Fl = (double)c1.sgn, Fpl = c1.f * Fl;
     double F = Fl, Fp = Fpl;
     double S = 0.0, R = 1.0;
-    for (int j = (l + 3) / 4 - 1; j >= 0; --j) {
-        coulomb_sr(4 * j + 1 + g.c, eta, rho, &S, &R);
-#pragma unroll
-        for (int u = 3; u >= 0; --u) {
+    for (int j = (l + W - 1) / W - 1; j >= 0; --j) {
+        coulomb_sr(W * j + 1 + g.c, eta, rho, &S, &R);
+        for (int u = min(W - 1, l - W * j - 1); u >= 0; --u) {
             const double SL = g.get(S, u), RL = g.get(R, u);
-            if (4 * j + 1 + u > l) continue;
             const double Fm = (SL * F + Fp) / RL;
             Fp = SL * Fm - RL * F;
             F = Fm;
@@ -977,12 +1025,10 @@ __device__ int open_channel_x4(const Quad &g, int l, double eps, double z, doubl
     const double scale = F0 / F;
     double G = scale * (Fp - p * F) / q;
     double Gp = p * G - q * F0;
-    for (int j = 0; 4 * j < l; ++j) {
-        if (j > 0) coulomb_sr(4 * j + 1 + g.c, eta, rho, &S, &R);   // j = 0: still there
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
+    for (int j = 0; W * j < l; ++j) {
+        if (j > 0) coulomb_sr(W * j + 1 + g.c, eta, rho, &S, &R);   // j = 0: still there
+        for (int u = 0; u < min(W, l - W * j); ++u) {
             const double S1 = g.get(S, u), R1 = g.get(R, u);
-            if (4 * j + 1 + u > l) continue;
             const double Gn = (S1 * G - Gp) / R1;
             Gp = R1 * G - S1 * Gn;
             G = Gn;
@@ -996,7 +1042,7 @@ __device__ int open_channel_x4(const Quad &g, int l, double eps, double z, doubl
     return 1;
 }
 
-template <bool MQDT> __device__ int closed_channel_x4(const Quad &g, int l, double eps, double z, double a, double *y)
+template <bool MQDT, int W> __device__ int closed_channel_xn(const Lanes<W> &g, int l, double eps, double z, double a, double *y)
 {
     const double kap = sqrt(-eps);
     const double nu = z / kap;
@@ -1006,7 +1052,7 @@ template <bool MQDT> __device__ int closed_channel_x4(const Quad &g, int l, doub
         L0 = L0 < 0 ? 0 : (L0 > l ? l : L0);
     }
     double yy;
-    if (!cf2_closed_x4<MQDT>(g, L0, nu, kap, a, &yy)) return 0;
+    if (!cf2_closed_xn<MQDT>(g, L0, nu, kap, a, &yy)) return 0;
     for (int L = L0; L < l; ++L) {
         const double L1 = L + 1.0;
         const double T = L1 / a - z / L1;
@@ -1017,26 +1063,27 @@ template <bool MQDT> __device__ int closed_channel_x4(const Quad &g, int l, doub
     return 1;
 }
 
-// One pair per four lanes; pairs (grid order, energy fastest) or those of a
+// One pair per W lanes; pairs (grid order, energy fastest) or those of a
 // list (deep != 0: the deep list, else all but the listed ones). Closed pairs
 // of the quantum-defect set need the regular solution's series in
 // double-double as well, one lane's work: the block collects them, one to a
 // thread of its first warp.
-template <bool MQDT>
-__global__ void __launch_bounds__(X4_BS)
-    chanfn_x4_kernel(PwDev pw, const double *__restrict__ E, int nE, Opts o, ChanFn *__restrict__ out,
+template <bool MQDT, int W>
+__global__ void __launch_bounds__(XN_BS)
+    chanfn_xn_kernel(PwDev pw, const double *__restrict__ E, int nE, Opts o, ChanFn *__restrict__ out,
                      int *__restrict__ status, const int *__restrict__ deep_count, const int *__restrict__ deep_list)
 {
-    __shared__ double ys[X4_PAIRS];
-    __shared__ int todo[X4_PAIRS];
-    const Quad g;
-    const int slot = threadIdx.x >> 2;
+    constexpr int PAIRS = XN_BS / W;
+    __shared__ double ys[PAIRS];
+    __shared__ int todo[PAIRS];
+    const Lanes<W> g;
+    const int slot = threadIdx.x / W;
     const int n = pw.n;
-    long long idx = (long long)blockIdx.x * X4_PAIRS + slot;
+    long long idx = (long long)blockIdx.x * PAIRS + slot;
     bool in = idx < (long long)nE * n;
     if (deep_list) {
         const int cnt = *deep_count;
-        if (cnt > CHANFN_DEEP_CAP || (long long)blockIdx.x * X4_PAIRS >= cnt) return;
+        if (cnt > CHANFN_DEEP_CAP || (long long)blockIdx.x * PAIRS >= cnt) return;
         in = idx < cnt;
         if (in) idx = deep_list[idx];
     }
@@ -1053,11 +1100,11 @@ __global__ void __launch_bounds__(X4_BS)
         if (fabs(eps) < o.eps_thr) {
             bad = RM_ETHRESHOLD;
         } else if (eps > 0.0) {
-            if (open_channel_x4(g, l, eps, z, a, &r.s, &r.sp, &r.gh, &r.ghp)) r.kind = CH_OPEN;
+            if (open_channel_xn(g, l, eps, z, a, &r.s, &r.sp, &r.gh, &r.ghp)) r.kind = CH_OPEN;
             else bad = RM_ECF_NOCONV;
         } else {
             double y;
-            if (!closed_channel_x4<MQDT>(g, l, eps, z, a, &y)) {
+            if (!closed_channel_xn<MQDT>(g, l, eps, z, a, &y)) {
                 bad = RM_ECF_NOCONV;
             } else {
                 const double nrm = 1.0 / sqrt(1.0 + (a * y) * (a * y));
@@ -1081,7 +1128,7 @@ __global__ void __launch_bounds__(X4_BS)
     }
     if constexpr (MQDT) {
         __syncthreads();
-        if (threadIdx.x >= X4_PAIRS || todo[threadIdx.x] < 0) return;
+        if (threadIdx.x >= PAIRS || todo[threadIdx.x] < 0) return;
         const int at = todo[threadIdx.x];
         const int e2 = at / n, i2 = at - e2 * n;
         const double eps2 = E[e2] - pw.e_thr[i2], y = ys[threadIdx.x];
@@ -1446,6 +1493,15 @@ cudaError_t launch_closed_table(const PwDev &pw, double *coef, unsigned char *ns
     return cudaGetLastError();
 }
 
+template <int W>
+static void launch_xn(const PwDev &pw, const double *E, int nE, const Opts &o, int mqdt, ChanFn *cf, int *status,
+                      const int *deep_count, const int *deep_list, long long pairs, cudaStream_t s)
+{
+    const unsigned grid = (unsigned)((pairs + XN_BS / W - 1) / (XN_BS / W));
+    if (mqdt) chanfn_xn_kernel<true, W><<<grid, XN_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_count, deep_list);
+    else chanfn_xn_kernel<false, W><<<grid, XN_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_count, deep_list);
+}
+
 static bool no_tables(const PwDev &pw) { return !pw.thr && !pw.otab && !pw.ctab; }
 
 cudaError_t launch_chanfn(const PwDev &pw, const double *E, int nE, const Opts &o, int mqdt,
@@ -1454,9 +1510,8 @@ cudaError_t launch_chanfn(const PwDev &pw, const double *E, int nE, const Opts &
     const long long total = (long long)nE * pw.n;
     if (total == 0) return cudaSuccess;
     if (no_tables(pw)) {
-        const unsigned grid4 = (unsigned)((total + X4_PAIRS - 1) / X4_PAIRS);
-        if (mqdt) chanfn_x4_kernel<true><<<grid4, X4_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_ws, nullptr);
-        else chanfn_x4_kernel<false><<<grid4, X4_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_ws, nullptr);
+        if (total <= XN_W8_PAIRS) launch_xn<8>(pw, E, nE, o, mqdt, cf, status, deep_ws, nullptr, total, s);
+        else launch_xn<4>(pw, E, nE, o, mqdt, cf, status, deep_ws, nullptr, total, s);
         return cudaGetLastError();
     }
     const unsigned grid = (unsigned)((total + CHANFN_BS - 1) / CHANFN_BS);
@@ -1484,10 +1539,8 @@ cudaError_t launch_chanfn_deep(const PwDev &pw, const double *E, int nE, const O
                                int *status, const int *deep_ws, cudaStream_t s)
 {
     if ((long long)nE * pw.n == 0) return cudaSuccess;
-    if (no_tables(pw)) {
-        const unsigned grid4 = (CHANFN_DEEP_CAP + X4_PAIRS - 1) / X4_PAIRS;
-        if (mqdt) chanfn_x4_kernel<true><<<grid4, X4_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_ws, deep_ws + 1);
-        else chanfn_x4_kernel<false><<<grid4, X4_BS, 0, s>>>(pw, E, nE, o, cf, status, deep_ws, deep_ws + 1);
+    if (no_tables(pw)) {   // few pairs, the deepest of all
+        launch_xn<8>(pw, E, nE, o, mqdt, cf, status, deep_ws, deep_ws + 1, CHANFN_DEEP_CAP, s);
         return cudaGetLastError();
     }
     const unsigned grid = (CHANFN_DEEP_CAP + 63) / 64;

@@ -1,4 +1,4 @@
-"""Channel functions without tables (four lanes per pair, csrc/channel_functions.cu): a pair's values do not depend
+"""Channel functions without tables (four or eight lanes per pair, csrc/channel_functions.cu): a pair's values do not depend
 on which pairs share its warp, its block or its list. All energies in one call against each alone, to the bit: pair
 counts around a block of 32, ladder lengths around a chunk of four l, fractions of very different depths side by
 side, pairs deep enough for the list, z = 0 on both sides of the distance from which its vanishing fractions are not
@@ -43,3 +43,22 @@ def test_alone_and_together(n, m, z, ls):
             assert np.isfinite(whole).all() and whole.any()
             for e in range(m):
                 assert np.array_equal(whole[e], f(E[e:e + 1])[0]), e
+
+
+@pytest.mark.parametrize("z", [0.0, 2.0])
+def test_eight_lanes_against_four(z):
+    """More than 16384 pairs take four lanes each, fewer eight: the same bits either way."""
+    n, m = 9, 2400
+    pw = synth.random_pw(5, n, 30, z=z, a=15.0, e_max=1.5, l_max=12)
+    E = np.sort(np.random.default_rng(1).uniform(0.02, 2.5, m))
+    with rmgb.Context(channel_tables=0) as ctx:
+        ctx.load_pw(0, pw)
+        got = []
+        for parts in (1, 2):
+            K = torch.zeros((m, n, n), dtype=torch.float64, device="cuda")
+            for mode in (0, 1):
+                for x, k in zip(np.split(E, parts), torch.split(K, m // parts)):
+                    ctx.solve_energies(0, x, mode, K_out=k)
+                    ctx.collision_strengths(reset=True)
+                got.append(K.cpu().numpy())
+        assert np.array_equal(got[0], got[2]) and np.array_equal(got[1], got[3])
