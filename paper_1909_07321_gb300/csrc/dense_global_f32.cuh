@@ -145,21 +145,31 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long k)
 
 // ---- real blocked LU ---------------------------------------------------------
 
+// Prefetch into L2 of the line at p.
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Rows [rlo, rhi) (stored from rstore; rlo a multiple of 4), columns
 // [c_lo, w): C += Lp x U, Lp the column-major panel of PB columns (stride
 // npad) holding the negated multipliers, U = rows [u0, u0 + PB) of M (final,
 // zero from column w to ld). Strips of 128 columns, their U copied
 // asynchronously into two shared buffers in turn (one barrier per strip);
-// thread (ty, tx) = (tid / 16, tid % 16) takes rows 4 ty .. 4 ty + 3 of each
-// tile of NTH / 4 rows and columns 4 tx .. 4 tx + 3 and 64 + 4 tx .. 64 + 4 tx
-// + 3 (a quarter-warp's float4 reads of U hit distinct banks). The C tile
-// after the current one, the next strip's first at a strip's end, is on its
-// way into registers while one is updated.
-template <int PB, int NTH>
+// thread (ty, tx) = (tid / 16, tid % 16) takes rows TI ty .. TI ty + TI - 1 of
+// each tile of TI NTH / 16 rows and columns 4 tx .. 4 tx + 3 and 64 + 4 tx ..
+// 64 + 4 tx + 3 (a quarter-warp's float4 reads of U hit distinct banks). The C
+// tile after the current one, the next strip's first at a strip's end, is on
+// its way meanwhile. Shared memory delivers 128 bytes a clock to a warp's
+// lanes, broadcast or not, and bounds the product: TI = 4 reads 48 bytes for
+// 32 FMAs and holds the next tile in registers, TI = 8 reads 64 for 64 and has
+// only L2 for the next tile. TI = 8 from 513 unknowns on (two panel rows a
+// thread, 512 threads): the solve of 152 systems of 513 open channels 8.96 ->
+// 8.39 ms, of 640 13.2 -> 12.4, of 1000 43.3 -> 41.8; below, where a tile of
+// 256 rows is most of the matrix, the elimination is 4-7 % slower with it.
+template <int PB, int NTH, int TI>
 __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int rstore, int c_lo, int w, const float *Lp,
                                int npad, float *Us)
 {
-    constexpr int TR = NTH / 4;   // rows per tile
+    constexpr int TR = TI * NTH / 16;   // rows per tile
+    constexpr bool REGS = TI == 4;     // the next tile in registers
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int nstrip = (w - c_lo + UW - 1) / UW;
     auto stage = [&](int s, float *buf) {
@@ -169,9 +179,9 @@ __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int r
             cp_async16(buf + k * (UW + 4) + j4, M + (size_t)(u0 + k) * ld + min(c, ld - 4), c < ld);
         }
     };
-    auto load = [&](int rb, int c0, unsigned long long (&v)[4][4]) {
+    auto load = [&](int rb, int c0, unsigned long long (&v)[TI][4]) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < TI; ++i) {
             const int r = rb + i;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -184,9 +194,9 @@ __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int r
         }
     };
     stage(0, Us);
-    unsigned long long acc[4][4], nxt[4][4];
-    const int rb0 = rlo + 4 * ty;
-    load(rb0, c_lo, acc);
+    unsigned long long acc[TI][4], nxt[REGS ? TI : 1][4];
+    const int rb0 = rlo + TI * ty;
+    if constexpr (REGS) load(rb0, c_lo, acc);
     for (int s = 0; s < nstrip; ++s) {
         const float *cur = Us + (s & 1) * PB * (UW + 4);
         const int c0 = c_lo + s * UW;
@@ -196,24 +206,37 @@ __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int r
         int rb = rb0;
         for (int r0 = rlo; r0 < rhi; r0 += TR, rb += TR) {
             const bool last = r0 + TR >= rhi;
-            if (!last) load(rb + TR, c0, nxt);
-            else if (s + 1 < nstrip) load(rb0, c0 + UW, nxt);
-            if (rb < rhi) {   // reads of Lp past rhi stay within the panel and feed rows that are not stored
-#pragma unroll 4
+            if constexpr (REGS) {
+                if (!last) load(rb + TR, c0, nxt);
+                else if (s + 1 < nstrip) load(rb0, c0 + UW, nxt);
+            } else {
+                load(rb, c0, acc);
+                // half a row's 128 columns a lane: two lines of 128 bytes
+                const int rn = (last ? rb0 : rb + TR) + (tx >> 1), cn = (last ? c0 + UW : c0) + 64 * (tx & 1);
+                if (rn < rhi && cn < ld) prefetch_l2(M + (size_t)rn * ld + cn);
+                if (rn < rhi && cn + 32 < ld) prefetch_l2(M + (size_t)rn * ld + cn + 32);
+            }
+            if (rb < rhi) {   // reads of Lp past rhi stay in shared memory and feed rows that are not stored
+#pragma unroll (REGS ? 4 : 2)
                 for (int k = 0; k < PB; ++k) {
-                    const float4 a4 = *reinterpret_cast<const float4 *>(Lp + k * npad + rb);
+                    float av[TI];
+#pragma unroll
+                    for (int i = 0; i < TI; i += 4) {
+                        const float4 q = *reinterpret_cast<const float4 *>(Lp + k * npad + rb + i);
+                        av[i] = q.x, av[i + 1] = q.y, av[i + 2] = q.z, av[i + 3] = q.w;
+                    }
                     const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(cur + k * (UW + 4) + 4 * tx);
                     const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(cur + k * (UW + 4) + 64 + 4 * tx);
-                    const unsigned long long a[4] = {pack2(a4.x, a4.x), pack2(a4.y, a4.y), pack2(a4.z, a4.z),
-                                                     pack2(a4.w, a4.w)};
                     const unsigned long long b[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                    for (int i = 0; i < TI; ++i) {
+                        const unsigned long long a = pack2(av[i], av[i]);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(a[i], b[j], acc[i][j]);
+                        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(a, b[j], acc[i][j]);
+                    }
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < TI; ++i) {
                     const int r = rb + i;
                     if (r >= rhi || r < rstore) continue;
 #pragma unroll
@@ -225,10 +248,12 @@ __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int r
                     }
                 }
             }
+            if constexpr (REGS) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < TI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = nxt[i][j];
+                    for (int j = 0; j < 4; ++j) acc[i][j] = nxt[i][j];
+            }
         }
     }
     __syncthreads();
@@ -446,6 +471,7 @@ template <int PB, int NTH, int RPT>
 __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int row_lo, float *smem)
 {
     constexpr int NWARP = NTH / 32;
+    constexpr int TI = RPT == 2 ? 8 : 4;   // rows of a thread in the updates
     const int tid = threadIdx.x;
     const int npad = lu_npad(n);
     float *Lp = smem;
@@ -521,7 +547,7 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 if (j < kb) M[(size_t)(k0 + j) * ld + c] = x[j];
         }
         __syncthreads();
-        if (k0 + kb < n) lu_update_rows<PB, NTH>(M, ld, k0, k0 + kb, n, k0 + kb, k0 + kb, w, Lp, npad, Us);
+        if (k0 + kb < n) lu_update_rows<PB, NTH, TI>(M, ld, k0, k0 + kb, n, k0 + kb, k0 + kb, w, Lp, npad, Us);
     }
     // back-substitution of rows [row_lo, n) for the right-hand sides
     const int rs = row_lo & ~3;
@@ -562,7 +588,7 @@ __device__ bool lu32_factor_solve(float *M, int ld, int n, int w, int rhs, int r
                 if (j < tb) M[(size_t)(t0 + j) * ld + c] = x[j];
         }
         __syncthreads();
-        if (t0 > row_lo) lu_update_rows<PB, NTH>(M, ld, t0, rs, t0, row_lo, rhs, w, Lp, npad, Us);
+        if (t0 > row_lo) lu_update_rows<PB, NTH, TI>(M, ld, t0, rs, t0, row_lo, rhs, w, Lp, npad, Us);
         t1 = t0;
     }
     return true;
