@@ -722,26 +722,32 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
             for (int k = 0; k < PB / 2; ++k)
                 Lp[(kh + k) * npz + i] = (kh + k < kb) ? unpack2(P[k]) : make_float2(0.f, 0.f);
         }
-        // Z_ij -= P_i Z_Kj for i, j outside K, i <= j, 64 columns at a time; the
+        // Z_ij -= P_i Z_Kj for i, j outside K, i <= j, 64 columns at a time (the
+        // first strip is the one with fewer, where there are the fewest rows:
+        // 512 systems of 150 / 200 / 260 open channels .670, 1.28, 2.43 ms with it
+        // last, .638, 1.14, 2.20 so); the
         // next strip's Z_Kj and the next tile's Z_ij are on their way meanwhile.
         // A warp leaves out its 8 rows of a tile where they lie below the
         // strip's last column, and the strip's first half where they lie below
         // that: the solve of 152 systems of 290 open channels 2.33 -> 2.28 ms, of 513
         // 8.44 -> 7.95, of 640 12.5 -> 11.8, of 1000 41.9 -> 40.5.
         const int nstrip = (m + UWC - 1) / UWC;
+        const int w0 = ((m + 1) & ~1) - (nstrip - 1) * UWC;   // columns of strip 0
+        auto strip0 = [&](int s) { return s ? w0 + (s - 1) * UWC : 0; };
         float2 st[SPT];
         auto fetch = [&](int s) {   // strips left of K lie in columns of Z: k fastest there
-            const bool left = s * UWC < k0;
+            const int c0 = strip0(s);
+            const bool left = c0 < k0;
 #pragma unroll
             for (int u = 0; u < SPT; ++u) {
                 const int q = tid + u * NTH;
-                const int k = left ? q % PB : q / UWC, c = s * UWC + (left ? q / PB : q % UWC);
+                const int k = left ? q % PB : q / UWC, c = c0 + (left ? q / PB : q % UWC);
                 const bool in = k < kb && c < m && (c < k0 || c >= k0 + kb);
                 st[u] = in ? zu(Z, ldz, k0 + k, c) : make_float2(0.f, 0.f);
             }
         };
         auto put = [&](int s) {
-            const bool left = s * UWC < k0;
+            const bool left = strip0(s) < k0;
             Op *buf = Us + (LEAN ? 0 : (s & 1)) * PB * (UWC + 2);
 #pragma unroll
             for (int u = 0; u < SPT; ++u) {
@@ -753,7 +759,7 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
             }
         };
         auto zload = [&](int rb, int c0, unsigned long long (&v)[4][4]) {
-            const int r_end = min(m, c0 + UWC);
+            const int c_end = c0 ? c0 + UWC : w0, r_end = min(m, c_end);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = rb + i;
@@ -761,7 +767,7 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
                 for (int h = 0; h < 2; ++h) {
                     const int c = c0 + 32 * h + 2 * tx;
                     ulonglong2 q = make_ulonglong2(0ull, 0ull);
-                    if (r < r_end && c < ldz) q = *reinterpret_cast<const ulonglong2 *>(Z + (size_t)r * ldz + c);
+                    if (r < r_end && c < c_end) q = *reinterpret_cast<const ulonglong2 *>(Z + (size_t)r * ldz + c);
                     v[i][2 * h] = q.x;
                     v[i][2 * h + 1] = q.y;
                 }
@@ -769,7 +775,7 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
         };
         unsigned long long acc[4][4], nxt[4][4];
         // columns 32 H0 .. 63 of the strip cur at c0, rows rb .. rb + 3
-        auto update = [&](auto h0, const Op *cur, int c0, int rb) {
+        auto update = [&](auto h0, const Op *cur, int c0, int c_end, int rb) {
             constexpr int H0 = decltype(h0)::value;
 #pragma unroll 4
             for (int k = 0; k < PB; ++k) {
@@ -796,7 +802,7 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
 #pragma unroll
                 for (int h = H0; h < 2; ++h) {
                     const int c = c0 + 32 * h + 2 * tx;
-                    if (c < ldz)
+                    if (c < c_end)
                         *reinterpret_cast<ulonglong2 *>(Z + (size_t)r * ldz + c) =
                             make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
                 }
@@ -807,7 +813,7 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
         const int rb0 = ty * 4;
         zload(rb0, 0, acc);
         for (int s = 0; s < nstrip; ++s) {
-            const int c0 = s * UWC;
+            const int c0 = strip0(s), c_end = c0 ? c0 + UWC : w0;
             const Op *cur = Us + (LEAN ? 0 : (s & 1)) * PB * (UWC + 2);
             if (LEAN) {
                 __syncthreads();
@@ -815,15 +821,15 @@ __device__ bool zsweep_invert(float2 *Z, int ldz, int m, float2 *smem)
             }
             __syncthreads();   // strip s (and, the first time, the panel) is complete
             if (s + 1 < nstrip) fetch(s + 1);
-            const int r_end = min(m, c0 + UWC);   // row tiles starting past this are below the diagonal
+            const int r_end = min(m, c_end);   // row tiles starting past this are below the diagonal
             int rb = rb0;
             for (int r0 = 0; r0 < r_end; r0 += TR, rb += TR) {
                 const bool last = r0 + TR >= r_end;
                 if (!last) zload(rb + TR, c0, nxt);
-                else if (s + 1 < nstrip) zload(rb0, c0 + UWC, nxt);
+                else if (s + 1 < nstrip) zload(rb0, c_end, nxt);
                 const int rw = rb & ~7;   // the warp's first row
-                if (rw >= c0 + 32 && rb < r_end) update(std::integral_constant<int, 1>(), cur, c0, rb);
-                else if (rb < r_end) update(std::integral_constant<int, 0>(), cur, c0, rb);
+                if (rw >= c0 + 32 && rb < r_end) update(std::integral_constant<int, 1>(), cur, c0, c_end, rb);
+                else if (rb < r_end) update(std::integral_constant<int, 0>(), cur, c0, c_end, rb);
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
