@@ -161,10 +161,10 @@ __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefe
 // its way meanwhile. Shared memory delivers 128 bytes a clock to a warp's
 // lanes, broadcast or not, and bounds the product: TI = 4 reads 48 bytes for
 // 32 FMAs and holds the next tile in registers, TI = 8 reads 64 for 64 and has
-// only L2 for the next tile. TI = 8 from 513 unknowns on (two panel rows a
-// thread, 512 threads): the solve of 152 systems of 513 open channels 8.96 ->
-// 8.39 ms, of 640 13.2 -> 12.4, of 1000 43.3 -> 41.8; below, where a tile of
-// 256 rows is most of the matrix, the elimination is 4-7 % slower with it.
+// only L2 for the next tile. TI = 8 with two panel rows a thread: the solve of
+// 152 systems of 513 open channels 8.96 -> 8.39 ms, of 640 13.2 -> 12.4, of
+// 1000 43.3 -> 41.8, the elimination of 512 of 331 (256 threads) 2.13 -> 1.90;
+// with one row a thread, where a tile is most of the matrix, it is 2-7 % slower.
 template <int PB, int NTH, int TI>
 __device__ void lu_update_rows(float *M, int ld, int u0, int rlo, int rhi, int rstore, int c_lo, int w, const float *Lp,
                                int npad, float *Us)

@@ -1225,6 +1225,17 @@ int max_dyn_smem()
     return v;
 }
 
+int sm_count()
+{
+    static int v = [] {
+        int dev = 0, x = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&x, cudaDevAttrMultiProcessorCount, dev);
+        return x;
+    }();
+    return v;
+}
+
 template <class K> cudaError_t set_smem(K kern, size_t bytes)
 {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -1254,14 +1265,22 @@ cudaError_t launch_lu32(int n, int nE, const EnergyDims *dims, double *ws, int *
     return cudaGetLastError();
 }
 
-// A panel's rows in the registers of 256 threads (two CTAs per SM) up to 256
-// channels, of 512 up to 512 (203 unknowns: 1.11 ms per 912 systems; two rows
-// a thread on 256 threads are slower at 431, 3.89 against 3.44 ms per 456),
-// two rows a thread up to 1024; in shared memory above.
+// A panel's rows in the registers of its threads, one or two rows each, up to
+// 1024 channels; in shared memory above. A panel is a serial chain, so more
+// and smaller CTAs an SM overlap one's panel with another's update: four of
+// 128 threads up to 128 channels, two of 256 (8 x 8 tiles) up to 448, as soon
+// as there are more energies than SMs; fewer energies have a whole SM each
+// anyway and are done sooner by more threads. 1024 systems of 97 unknowns .324
+// ms with 256 threads, .218 with 128; 512 of 110 .223, .171; 152 of 64 .049,
+// .051. 512 of 290 1.79 with 512 threads, 1.45 with 256, of 331 2.25, 1.90, of
+// 431 4.16, 3.69, of 470 5.21, 5.23; 152 of 331 .567, .672.
 cudaError_t launch_lu32_any(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
                             cudaStream_t st)
 {
+    const bool many = nE > sm_count();
+    if (n <= 128 && many) return launch_lu32<32, 128, 1>(n, nE, dims, ws, status, order, st);
     if (n <= 256) return launch_lu32<32, 256, 1>(n, nE, dims, ws, status, order, st);
+    if (n <= 448 && many) return launch_lu32<32, 256, 2>(n, nE, dims, ws, status, order, st);
     if (n <= 512) return launch_lu32<32, 512, 1>(n, nE, dims, ws, status, order, st);
     if (n <= 1024) return launch_lu32<32, 512, 2>(n, nE, dims, ws, status, order, st);
     if (lu_pb(n) == 32) return launch_lu32<32, 512, 0>(n, nE, dims, ws, status, order, st);

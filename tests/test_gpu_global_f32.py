@@ -38,3 +38,24 @@ def test_against_fp64_solve(n, m, mode):
     off = np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)
     assert np.isfinite(off).all()
     assert np.median(off) <= max(n, 16) * 2.0 ** -18, off
+
+
+@pytest.mark.parametrize("n", [5, 97, 128, 257, 300, 448])
+def test_many_energies_as_few(n):
+    """More energies than SMs take smaller CTAs (up to 128 and 448 channels): the same bits."""
+    m = 2 * (torch.cuda.get_device_properties(0).multi_processor_count // 2 + 4)
+    pw = synth.random_pw(700 + n, n, n + 20, z=2.0, a=15.0, e_max=1.5, sigma=0.1)
+    E = np.linspace(0.11, 1.61, m) + 0.003
+    Ks, oms = [], []
+    for parts in (1, 2):
+        with rmgb.Context(precision=rmgb.RM_FP64, solve_precision=rmgb.RM_FP32, solver=rmgb.RM_SOLVER_LARGE) as ctx:
+            ctx.load_pw(0, pw)
+            K = torch.zeros((m, n, n), dtype=torch.float64, device="cuda")
+            om = []
+            for x, k in zip(np.split(E, parts), torch.split(K, m // parts)):
+                ctx.solve_energies(0, x, 0, K_out=k)
+                om.append(ctx.collision_strengths(reset=True))
+            Ks.append(K.cpu().numpy())
+            oms.append(np.concatenate(om))
+    assert np.array_equal(Ks[0], Ks[1])
+    assert np.array_equal(oms[0], oms[1])
