@@ -1268,19 +1268,20 @@ cudaError_t launch_lu32(int n, int nE, const EnergyDims *dims, double *ws, int *
 // A panel's rows in the registers of its threads, one or two rows each, up to
 // 1024 channels; in shared memory above. A panel is a serial chain, so more
 // and smaller CTAs an SM overlap one's panel with another's update: four of
-// 128 threads up to 128 channels, two of 256 (8 x 8 tiles) up to 448, as soon
-// as there are more energies than SMs; fewer energies have a whole SM each
-// anyway and are done sooner by more threads. 1024 systems of 97 unknowns .324
-// ms with 256 threads, .218 with 128; 512 of 110 .223, .171; 152 of 64 .049,
-// .051. 512 of 290 1.79 with 512 threads, 1.45 with 256, of 331 2.25, 1.90, of
-// 431 4.16, 3.69, of 470 5.21, 5.23; 152 of 331 .567, .672.
+// 128 threads up to 128 channels, two of 256 (8 x 8 tiles) up to 448, where
+// there are more energies than the larger CTAs have room for at once; fewer
+// are done sooner by more threads (304 of 97: .404 ms with the sweep, .420 with
+// 128). 1024 systems of 97 unknowns .324 ms with 256 threads, .218 with 128;
+// 512 of 110 .223, .171; 152 of 64 .049, .051. 512 of 290 1.79 with 512
+// threads, 1.45 with 256, of 331 2.25, 1.90, of 431 4.16, 3.69, of 470 5.21,
+// 5.23; 152 of 331 .567, .672.
 cudaError_t launch_lu32_any(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
                             cudaStream_t st)
 {
-    const bool many = nE > sm_count();
-    if (n <= 128 && many) return launch_lu32<32, 128, 1>(n, nE, dims, ws, status, order, st);
+    const int sms = sm_count();
+    if (n <= 128 && nE > 2 * sms) return launch_lu32<32, 128, 1>(n, nE, dims, ws, status, order, st);
     if (n <= 256) return launch_lu32<32, 256, 1>(n, nE, dims, ws, status, order, st);
-    if (n <= 448 && many) return launch_lu32<32, 256, 2>(n, nE, dims, ws, status, order, st);
+    if (n <= 448 && nE > sms) return launch_lu32<32, 256, 2>(n, nE, dims, ws, status, order, st);
     if (n <= 512) return launch_lu32<32, 512, 1>(n, nE, dims, ws, status, order, st);
     if (n <= 1024) return launch_lu32<32, 512, 2>(n, nE, dims, ws, status, order, st);
     if (lu_pb(n) == 32) return launch_lu32<32, 512, 0>(n, nE, dims, ws, status, order, st);
@@ -1299,9 +1300,10 @@ cudaError_t launch_zsweep(int n, int nE, const EnergyDims *dims, double *ws, int
 }
 
 // Two CTAs of 256 threads per SM while their shared memory fits (up to 512
-// channels: 300 open ones 2.30 against 2.76 ms per 456 systems on 512
-// threads; 500 open 6.80 against 6.57 ms per 304). The pivots per block (16,
-// above 1733 channels 8) decide the rounding and do not depend on this.
+// channels: 260 open ones 2.20 against 2.64 ms per 512 systems on 512
+// threads, 400 open 6.15 against 6.79; 500 open 6.73 against 6.06 per 304).
+// The pivots per block (16, above 1733 channels 8) decide the rounding and do
+// not depend on this.
 cudaError_t launch_zsweep_any(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order,
                               cudaStream_t st)
 {

@@ -42,8 +42,9 @@ def test_against_fp64_solve(n, m, mode):
 
 @pytest.mark.parametrize("n", [5, 97, 128, 257, 300, 448])
 def test_many_energies_as_few(n):
-    """More energies than SMs take smaller CTAs (up to 128 and 448 channels): the same bits."""
-    m = 2 * (torch.cuda.get_device_properties(0).multi_processor_count // 2 + 4)
+    """More energies than fit at once take smaller CTAs (up to 128 and 448 channels): the same bits."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    m = 2 * ((2 * sms if n <= 128 else sms) // 2 + 4)
     pw = synth.random_pw(700 + n, n, n + 20, z=2.0, a=15.0, e_max=1.5, sigma=0.1)
     E = np.linspace(0.11, 1.61, m) + 0.003
     Ks, oms = [], []
