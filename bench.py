@@ -924,7 +924,7 @@ def run_ours(args, rank, world, local_rank):
     form_ach = form_flops / (per_launch_ms(rmgb.RM_PH_FORM) * 1e-3) / 1e12
     if prec == 0:
         form_roof = {"bound": "alu", "achieved": form_ach, "peak": fp64_peak, "unit": "TFLOP/s",
-                     "frac": form_ach / fp64_peak, "traffic": None, "kernel": "form_r_tiled (FP64)",
+                     "frac": form_ach / fp64_peak, "traffic": None, "kernel": "form_r_packed (FP64)",
                      "peak_source": "FP64 4 flop/clk/SM x 152 SMs at the sampled SM clock"}
     else:
         tpk = peaks["bf16_tflops"] if prec == 2 else peaks["bf16_tflops"] / 2.0
