@@ -198,6 +198,7 @@ struct Lane {
     std::vector<cudaEvent_t> piece_ev;
     std::vector<int> piece_end;
     int n_pieces = 0;
+    bool want_pieces = true;   // the last call was a blocking read-out, or there was none
     // workspace
     DevBuf wsE, wsCf, wsR, wsStatus, wsMq, wsDh, wsDl, wsErr, wsL, wsPart, wsDeep, wsNear, wsEhl;
     // coarse-mesh interpolation: node energies, statuses + orders, K_u, S_u, fine plan
@@ -1023,7 +1024,10 @@ int pieces_of(int nE, int ntri)
 }
 
 // Whether the lane's next solve may note its pieces: not while its stream is
-// being captured (an event recorded there cannot be waited for outside).
+// being captured (an event recorded there cannot be waited for outside), and
+// only right after a blocking read-out or as the lane's first: where Omega
+// stays on the device or is read out asynchronously the pieces' ends would
+// cost 2 % for nothing (20000 energies of 64 channels 3.82 -> 3.90 ms).
 bool may_note_pieces(Lane *ln)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -1031,7 +1035,10 @@ bool may_note_pieces(Lane *ln)
         cudaGetLastError();
         return false;
     }
-    return st == cudaStreamCaptureStatusNone;
+    if (st != cudaStreamCaptureStatusNone) return false;
+    const bool want = ln->want_pieces;
+    ln->want_pieces = false;
+    return want;
 }
 
 // The rows before `end` are final once the work enqueued so far is done.
@@ -1406,6 +1413,7 @@ int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset
     CK(cudaStreamSynchronize(ln->stream));
     int rc = check_device_flag(ctx, ln);
     if (rc) return rc;
+    if (omega_out) ln->want_pieces = true;
     if (reset) {
         ln->n_pieces = 0;
         ln->grid_nE = ln->grid_nlev = ln->grid_ntri = 0;
@@ -1472,6 +1480,7 @@ extern "C" int rm_collision_strengths_async(rm_ctx *ctx, double *omega_out, int 
     const int crc = copy_stream(ctx, ln);
     if (crc) return crc;
     ln->n_pieces = 0;
+    ln->want_pieces = false;
     const size_t bytes = (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double);
     const int cur = ln->omega_cur;
     CK(cudaEventRecord(ln->ev_solved, ln->stream));
