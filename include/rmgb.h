@@ -303,7 +303,12 @@ int rm_qdt_plan_inspect(int n_ch, const double *e_thr, double z, int n_poles, co
 /* Copies the accumulated collision strengths to omega_out (host,
  * [n_E][n_levels*(n_levels+1)/2], upper triangle row-wise: (I, J), I <= J,
  * at I*n_levels - I*(I-1)/2 + (J - I)); entries of levels closed at E are 0.
- * Synchronises the stream. reset != 0 zeroes the accumulator and forgets the
+ * Synchronises the stream. The copy follows everything enqueued on the stream
+ * before the call, the caller's own work included. Only on a stream that the
+ * context owns (rm_opts.stream NULL, lanes 1 and up) and that rm_lane_stream
+ * never returned, where there can be no such work, are rows copied to
+ * omega_out as soon as they are final, beside the solve of later
+ * ones. reset != 0 zeroes the accumulator and forgets the
  * grid. omega_out may be NULL (reset only). Errors: RM_EINVAL (no grid yet),
  * RM_ECUDA. */
 int rm_collision_strengths(rm_ctx *ctx, double *omega_out, int reset);
@@ -433,7 +438,8 @@ int rm_lane_query(rm_ctx *ctx, int lane);
 /* Waits for the lane's stream. */
 int rm_lane_sync(rm_ctx *ctx, int lane);
 
-/* The lane's cudaStream_t (NULL for a bad lane or context). */
+/* The lane's cudaStream_t (NULL for a bad lane or context). From then on the
+ * lane's read-outs copy after all work on the stream, as on a caller's. */
 void *rm_lane_stream(rm_ctx *ctx, int lane);
 
 /* Sizes lane `lane`'s workspace and Omega accumulator for a solve of n_E

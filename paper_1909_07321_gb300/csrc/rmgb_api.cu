@@ -180,6 +180,7 @@ namespace {
 struct Lane {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    bool handed_out = false;   // rm_lane_stream has given the stream to the caller
     // grid and Omega accumulator
     int grid_nE = 0, grid_nlev = 0, grid_ntri = 0;
     std::vector<double> grid_host;
@@ -1023,20 +1024,20 @@ int pieces_of(int nE, int ntri)
     return (int)std::min<size_t>(std::max<size_t>(p, 1), MAX_PIECES);
 }
 
-// Whether the lane's next solve may note its pieces: not while its stream is
-// being captured (an event recorded there cannot be waited for outside), and
-// only right after a blocking read-out or as the lane's first: where Omega
-// stays on the device or is read out asynchronously the pieces' ends would
-// cost 2 % for nothing (20000 energies of 64 channels 3.82 -> 3.90 ms).
+// A piece's copy follows its event alone and would overtake whatever the
+// caller enqueues between the solve and the read-out (an upload out of
+// omega_out, a replay of a solve that it captured): pieces are for streams on
+// which nothing of the caller's can be, those that the context created and
+// rm_lane_stream never gave out.
+bool private_stream(const Lane *ln) { return ln->own_stream && !ln->handed_out; }
+
+// Whether the lane's next solve may note its pieces: only right after a
+// blocking read-out or as the lane's first: where Omega stays on the device or
+// is read out asynchronously the pieces' ends would cost 2 % for nothing
+// (20000 energies of 64 channels 3.82 -> 3.90 ms).
 bool may_note_pieces(Lane *ln)
 {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ln->stream, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (st != cudaStreamCaptureStatusNone) return false;
-    const bool want = ln->want_pieces;
+    const bool want = ln->want_pieces && private_stream(ln);
     ln->want_pieces = false;
     return want;
 }
@@ -1391,7 +1392,7 @@ int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset
         return fail(ctx, RM_EINVAL, "no energy grid registered yet");
     }
     const size_t bytes = (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double);
-    if (omega_out && ln->n_pieces > 1 && ln->piece_end[ln->n_pieces - 1] == ln->grid_nE) {
+    if (omega_out && private_stream(ln) && ln->n_pieces > 1 && ln->piece_end[ln->n_pieces - 1] == ln->grid_nE) {
         int rc = copy_stream(ctx, ln);
         if (rc) return rc;
         cudaError_t err = cudaSuccess;
@@ -1467,6 +1468,7 @@ extern "C" int rm_lane_sync(rm_ctx *ctx, int lane)
 extern "C" void *rm_lane_stream(rm_ctx *ctx, int lane)
 {
     if (!ctx || lane < 0 || lane >= (int)ctx->lanes.size()) return nullptr;
+    ctx->lanes[lane].handed_out = true;
     return ctx->lanes[lane].stream;
 }
 
