@@ -306,8 +306,8 @@ int rm_qdt_plan_inspect(int n_ch, const double *e_thr, double z, int n_poles, co
  * Synchronises the stream. The copy follows everything enqueued on the stream
  * before the call, the caller's own work included. Only on a stream that the
  * context owns (rm_opts.stream NULL, lanes 1 and up) and that rm_lane_stream
- * never returned, where there can be no such work, are rows copied to
- * omega_out as soon as they are final, beside the solve of later
+ * never returned, where there can be no such work, are rows copied into
+ * page-locked omega_out as soon as they are final, beside the solve of later
  * ones. reset != 0 zeroes the accumulator and forgets the
  * grid. omega_out may be NULL (reset only). Errors: RM_EINVAL (no grid yet),
  * RM_ECUDA. */

@@ -199,7 +199,7 @@ struct Lane {
     std::vector<cudaEvent_t> piece_ev;
     std::vector<int> piece_end;
     int n_pieces = 0;
-    bool want_pieces = true;   // the last call was a blocking read-out, or there was none
+    bool want_pieces = true;   // the last call was a blocking read-out into page-locked memory, or there was none
     // workspace
     DevBuf wsE, wsCf, wsR, wsStatus, wsMq, wsDh, wsDl, wsErr, wsL, wsPart, wsDeep, wsNear, wsEhl;
     // coarse-mesh interpolation: node energies, statuses + orders, K_u, S_u, fine plan
@@ -291,6 +291,16 @@ bool is_device_ptr(const void *p)
         return false;
     }
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+bool is_page_locked(const void *p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeHost;
 }
 
 bool finite_all(const double *x, size_t n)
@@ -1032,9 +1042,11 @@ int pieces_of(int nE, int ntri)
 bool private_stream(const Lane *ln) { return ln->own_stream && !ln->handed_out; }
 
 // Whether the lane's next solve may note its pieces: only right after a
-// blocking read-out or as the lane's first: where Omega stays on the device or
-// is read out asynchronously the pieces' ends would cost 2 % for nothing
-// (20000 energies of 64 channels 3.82 -> 3.90 ms).
+// blocking read-out into page-locked memory or as the lane's first. Where
+// Omega stays on the device or is read out asynchronously the pieces' ends
+// would cost 2 % for nothing (20000 energies of 64 channels 3.82 -> 3.90 ms),
+// and pageable memory takes pieces far more slowly than one copy (24 requests
+// of 50 to 1492 channels on one lane, 19 GB: 4.0 to 5.0 s, one copy each 0.7).
 bool may_note_pieces(Lane *ln)
 {
     const bool want = ln->want_pieces && private_stream(ln);
@@ -1392,7 +1404,8 @@ int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset
         return fail(ctx, RM_EINVAL, "no energy grid registered yet");
     }
     const size_t bytes = (size_t)ln->grid_nE * ln->grid_ntri * sizeof(double);
-    if (omega_out && private_stream(ln) && ln->n_pieces > 1 && ln->piece_end[ln->n_pieces - 1] == ln->grid_nE) {
+    const bool locked = omega_out && is_page_locked(omega_out);
+    if (locked && private_stream(ln) && ln->n_pieces > 1 && ln->piece_end[ln->n_pieces - 1] == ln->grid_nE) {
         int rc = copy_stream(ctx, ln);
         if (rc) return rc;
         cudaError_t err = cudaSuccess;
@@ -1414,7 +1427,7 @@ int collision_strengths_lane(rm_ctx *ctx, Lane *ln, double *omega_out, int reset
     CK(cudaStreamSynchronize(ln->stream));
     int rc = check_device_flag(ctx, ln);
     if (rc) return rc;
-    if (omega_out) ln->want_pieces = true;
+    if (omega_out) ln->want_pieces = locked;
     if (reset) {
         ln->n_pieces = 0;
         ln->grid_nE = ln->grid_nlev = ln->grid_ntri = 0;

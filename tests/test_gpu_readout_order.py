@@ -122,3 +122,38 @@ def test_on_a_stream_of_the_contexts_own(m, more, kind):
             solve(ctx, kind, 1, E)
             assert np.array_equal(ctx.collision_strengths(out), two)
             assert np.array_equal(ctx.collision_strengths(out, reset=True), two)
+
+
+def test_rows_beside_the_solve_only_into_page_locked_memory():
+    """Pageable memory takes many small copies several times more slowly than one, so a solve after a read-out into it
+    is not cut up: on the context's own stream it has the launches that it has on a caller's, and so once the stream
+    was asked for; after a read-out into page-locked memory it has more."""
+    m = 6100
+    E = synth.midpoint_grid(0.01, 2.5, m)
+    locked, pageable = pinned(m).numpy(), np.empty((m, TRI))
+
+    def launches(ctx, out):
+        """of the solve after a read-out into `out`"""
+        ctx.solve_energies(0, E)
+        ctx.collision_strengths(out, reset=True)
+        before = ctx.launch_count()
+        ctx.solve_energies(0, E)
+        n = ctx.launch_count() - before
+        ctx.collision_strengths(out, reset=True)
+        return n
+
+    with rmgb.Context(**MIXED) as ctx:
+        load(ctx)
+        whole = launches(ctx, locked)
+        assert launches(ctx, pageable) == whole
+    want = locked.copy()
+    with rmgb.Context(stream=0, **MIXED) as ctx:
+        load(ctx)
+        assert launches(ctx, pageable) == whole
+        assert np.array_equal(pageable, want)
+        assert launches(ctx, locked) > whole
+        assert np.array_equal(locked, want)
+        assert launches(ctx, pageable) == whole
+        ctx.lane_stream(0)
+        assert launches(ctx, locked) == whole
+        assert np.array_equal(locked, want)
