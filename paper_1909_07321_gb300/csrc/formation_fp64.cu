@@ -114,8 +114,7 @@ template <int PT, int TK, bool DIV>
 cudaError_t launch_packed(const PwDev &pw, const double *E, int nE, double *R, int nw, int ctas, cudaStream_t s)
 {
     const size_t smem = ((size_t)2 * pw.n * (TK + 1) + 2 * TK) * sizeof(double);
-    const cudaError_t e = cudaFuncSetAttribute(form_r_packed<PT, TK, DIV>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(form_r_packed<PT, TK, DIV>, smem);
     if (e != cudaSuccess) return e;
     form_r_packed<PT, TK, DIV><<<dim3(ctas, nE), nw * 32, smem, s>>>(pw, E, R);
     return cudaGetLastError();

@@ -413,8 +413,7 @@ cudaError_t launch_pair_variant(const void *D_hi, const void *D_lo, const void *
     const int n_tiles = n_mt * n_nt;
     const int grid = n_tiles < num_sms() ? n_tiles : num_sms();
     const size_t smem = (size_t)STAGES * PairTile<BN>::STAGE_BYTES + 1024 + 256;
-    cudaError_t e = cudaFuncSetAttribute(form_r_tc_kernel<KIND, BN, STAGES>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(form_r_tc_kernel<KIND, BN, STAGES>, smem);
     if (e != cudaSuccess) return e;
     form_r_tc_kernel<KIND, BN, STAGES><<<grid, NTHREADS, smem, s>>>(mDh, mDl, mPh, mPl, Rp, ldR, nE, n_pairs,
                                                                     n_kb, n_nt, n_tiles, err_flag, probe_ns);

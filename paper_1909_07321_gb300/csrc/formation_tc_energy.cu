@@ -571,14 +571,12 @@ cudaError_t launch_form_r_pe(int kind, int n, int Kpad, const float *W32, const 
     const long long grid = g.n_items < num_sms() ? g.n_items : num_sms();
     cudaError_t e;
     if (kind == TC_BF16X3) {
-        e = cudaFuncSetAttribute(form_r_pe_kernel<TC_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 PE_SMEM);
+        e = allow_smem(form_r_pe_kernel<TC_BF16X3>, PE_SMEM);
         if (e != cudaSuccess) return e;
         form_r_pe_kernel<TC_BF16X3><<<(unsigned)grid, PE_THREADS, PE_SMEM, s>>>(mh, ml, W32, D32, part, g,
                                                                                  err_flag, probe_ns);
     } else {
-        e = cudaFuncSetAttribute(form_r_pe_kernel<TC_TF32X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 PE_SMEM);
+        e = allow_smem(form_r_pe_kernel<TC_TF32X3>, PE_SMEM);
         if (e != cudaSuccess) return e;
         form_r_pe_kernel<TC_TF32X3><<<(unsigned)grid, PE_THREADS, PE_SMEM, s>>>(mh, ml, W32, D32, part, g,
                                                                                  err_flag, probe_ns);

@@ -706,22 +706,19 @@ cudaError_t launch_propagate(const PwDev &pw, const double *E, int nE, const dou
     if (nE == 0) return cudaSuccess;
     const size_t smem = propagate_smem(pw.n, lmax);
     if (pw.n <= PROP_SMALL_MAXN) {
-        cudaError_t err =
-            cudaFuncSetAttribute(propagate_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t err = allow_smem(propagate_small_kernel, smem);
         if (err != cudaSuccess) return err;
         const int G = prop_groups(pw.n);
         propagate_small_kernel<<<(nE + G - 1) / G, NT, smem, s>>>(pw, E, nE, A, lmax, r1, steps, Rp, status);
         return cudaGetLastError();
     }
     if (pw.n <= 32) {
-        cudaError_t err =
-            cudaFuncSetAttribute(propagate_kernel<256, 4, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t err = allow_smem(propagate_kernel<256, 4, 32>, smem);
         if (err != cudaSuccess) return err;
         propagate_kernel<256, 4, 32><<<nE, 256, smem, s>>>(pw, E, A, lmax, r1, steps, Rp, status);
         return cudaGetLastError();
     }
-    cudaError_t err =
-        cudaFuncSetAttribute(propagate_kernel<512, 8, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = allow_smem(propagate_kernel<512, 8, 64>, smem);
     if (err != cudaSuccess) return err;
     propagate_kernel<512, 8, 64><<<nE, 512, smem, s>>>(pw, E, A, lmax, r1, steps, Rp, status);
     return cudaGetLastError();

@@ -587,8 +587,7 @@ cudaError_t launch_qdt_s_from_k(int n, int n_nodes, const double *Ku, const int 
 {
     if (n_nodes == 0) return cudaSuccess;
     const size_t smem = qdt_s_smem(n);
-    cudaError_t e = cudaFuncSetAttribute(qdt_s_from_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = allow_smem(qdt_s_from_k_kernel, smem);
     if (e != cudaSuccess) return e;
     qdt_s_from_k_kernel<<<n_nodes, NTS, smem, s>>>(n, Ku, np_node, status, Su);
     return cudaGetLastError();
@@ -603,13 +602,13 @@ cudaError_t launch_qdt_fine(int iqdt, const PwDev &pw, const double *E, int nE, 
     cudaError_t e;
     if (iqdt == 2) {
         const size_t smem = (size_t)3 * pw.n * (pw.n + 1) * sizeof(double);
-        e = cudaFuncSetAttribute(qdt_fine_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(qdt_fine_kernel<2>, smem);
         if (e != cudaSuccess) return e;
         qdt_fine_kernel<2><<<nE, NT, smem, s>>>(pw, E, o, fine, Ku, Su, node_status, status, n_open_out, omega,
                                                 n_tri);
     } else {
         const size_t smem = (size_t)pw.n * (pw.n + 1) * sizeof(double2);
-        e = cudaFuncSetAttribute(qdt_fine_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(qdt_fine_kernel<1>, smem);
         if (e != cudaSuccess) return e;
         qdt_fine_kernel<1><<<nE, NT, smem, s>>>(pw, E, o, fine, Ku, Su, node_status, status, n_open_out, omega,
                                                 n_tri);

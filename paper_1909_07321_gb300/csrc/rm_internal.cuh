@@ -10,6 +10,25 @@
 
 namespace rmgb {
 
+// Lets `kern` be launched with `bytes` of dynamic shared memory. The limit
+// belongs to the kernel in the whole process, while each host thread may run a
+// context of its own: set to what one launch needs, it could be lowered by
+// another thread's smaller wave before that launch, which then failed. So it
+// is raised to the most the device allows and never lowered.
+template <class K> cudaError_t allow_smem(K kern, size_t bytes)
+{
+    cudaFuncAttributes at;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaFuncGetAttributes(&at, kern);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    most -= (int)at.sharedSizeBytes;
+    if (bytes > (size_t)most) return cudaErrorInvalidValue;
+    if (at.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Boundary data of one channel at one energy (step (b)).
 //   open (CH_OPEN):        (gh, ghp) = (c, c'),  (s, sp) = (s, s')   energy-normalised Coulomb
 //   closed (CH_CLOSED):    (gh, ghp) = (theta, theta') with theta^2 + (a theta')^2 = 1, s = sp = 0

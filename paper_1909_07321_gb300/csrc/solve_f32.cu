@@ -744,8 +744,7 @@ cudaError_t launch_tile(const PwDev &pw, const double *E, int nE, const ChanFn *
                         cudaStream_t s)
 {
     const size_t smem = ((size_t)tri_ld(pw.n) + (size_t)pw.n * pw.n) * sizeof(float);
-    cudaError_t err =
-        cudaFuncSetAttribute(solve_f32_kernel<TR, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = allow_smem(solve_f32_kernel<TR, TC>, smem);
     if (err != cudaSuccess) return err;
     solve_f32_kernel<TR, TC><<<nE, NT, smem, s>>>(pw, E, cf, R, status, K_out, n_open_out, omega, n_tri, deep_ws,
                                                   chanfn_deep_cap(), pass);

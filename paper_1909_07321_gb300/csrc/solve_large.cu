@@ -695,7 +695,7 @@ cudaError_t launch_lu64(int n, int nE, const LuJob *lu, int *status, cudaStream_
         return cudaGetLastError();
     }
     const size_t sm = l64_smem(n);
-    const cudaError_t err = cudaFuncSetAttribute(lu64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t err = allow_smem(lu64_kernel, sm);
     if (err != cudaSuccess) return err;
     lu64_kernel<<<nE, NTH, sm, st>>>(lu, status, n, l64_strip(n));
     return cudaGetLastError();
@@ -1236,11 +1236,6 @@ int sm_count()
     return v;
 }
 
-template <class K> cudaError_t set_smem(K kern, size_t bytes)
-{
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // Panel widths that fit shared memory for n channels (0: none fits).
 int lu_pb(int n)
 {
@@ -1259,7 +1254,7 @@ template <int PB, int NT, int RPT>
 cudaError_t launch_lu32(int n, int nE, const EnergyDims *dims, double *ws, int *status, const int *order, cudaStream_t st)
 {
     const size_t sm = f32d::lu_smem<PB, NT, RPT>(n);
-    const cudaError_t err = set_smem(lu32_kernel<PB, NT, RPT>, sm);
+    const cudaError_t err = allow_smem(lu32_kernel<PB, NT, RPT>, sm);
     if (err != cudaSuccess) return err;
     lu32_kernel<PB, NT, RPT><<<nE, NT, sm, st>>>(n, dims, ws, status, order);
     return cudaGetLastError();
@@ -1293,7 +1288,7 @@ cudaError_t launch_zsweep(int n, int nE, const EnergyDims *dims, double *ws, int
                           cudaStream_t st)
 {
     const size_t sm = f32d::z_smem<PB, LEAN>(n);
-    const cudaError_t err = set_smem(zsweep_kernel<PB, NT, LEAN>, sm);
+    const cudaError_t err = allow_smem(zsweep_kernel<PB, NT, LEAN>, sm);
     if (err != cudaSuccess) return err;
     zsweep_kernel<PB, NT, LEAN><<<nE, NT, sm, st>>>(n, dims, ws, status, order);
     return cudaGetLastError();

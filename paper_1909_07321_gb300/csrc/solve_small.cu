@@ -219,8 +219,7 @@ cudaError_t launch_solve_small(const PwDev &pw, const double *E, int nE, const C
     if (f32) return launch_solve_f32(pw, E, nE, cf, R, status, K_out, n_open_out, omega, n_tri, deep_ws, pass, s);
     const size_t smem = solve_small_smem(pw.n);
     const int cap = chanfn_deep_cap();
-    cudaError_t err =
-        cudaFuncSetAttribute(solve_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = allow_smem(solve_small_kernel, smem);
     if (err != cudaSuccess) return err;
     solve_small_kernel<<<nE, NT, smem, s>>>(pw, E, cf, R, status, K_out, n_open_out, omega, n_tri, mqdt ? 1 : 0,
                                             deep_ws, cap, pass, ku_out, ku_np);
