@@ -11,7 +11,7 @@
 namespace rmgb {
 namespace {
 
-// n <= PK_MAX_N: the packed pairs p = (i <= j) of one energy dealt out 32 to a
+// Where packed_wins(n): the packed pairs p = (i <= j) of one energy dealt out 32 to a
 // warp load, PT loads a warp, so that no FP64 FMA is spent on an entry that is
 // not stored. GB300 issues 2 FP64 FMAs per clock and SM, and everything else
 // (two shared loads per FMA, the staging) fits beside them; a 64 x 64 tile
@@ -26,7 +26,6 @@ namespace {
 // rows j read distinct banks), the next chunk's W and the chunk after that
 // one's d already on their way. Every entry is one chain of FMAs over
 // ascending poles.
-constexpr int PK_MAX_N = 1024;
 constexpr int PK_MAX_WARPS = 16;
 
 template <int PT, int TK, bool DIV>
@@ -120,34 +119,68 @@ cudaError_t launch_packed(const PwDev &pw, const double *E, int nE, double *R, i
     return cudaGetLastError();
 }
 
-// Loads per warp, warps and CTAs per energy: the least of CTAs x (warp-load
-// lanes + rows to be scaled), the FP64 work of a pole.
-cudaError_t launch_packed_any(const PwDev &pw, const double *E, int nE, double *R, cudaStream_t s)
+// Loads per warp, warps and CTAs per energy.
+struct PkPlan {
+    int pt, nw, ctas;
+};
+
+// From 32 channels on, the least of CTAs x (warp-load lanes + rows to be
+// scaled), the FP64 work of a pole.
+PkPlan pk_plan(int n)
 {
-    const int n = pw.n, nq = (tri_count(n) + 31) / 32;
-    int pt = 1, nw = 1, ctas = nq;
+    const int nq = (tri_count(n) + 31) / 32;
     if (n < 32) {
-        pt = nq <= 4 ? 1 : (nq <= 8 ? 2 : 4);
-        nw = (nq + pt - 1) / pt;
-        ctas = 1;
-    } else {
-        long long best = 0;
-        for (int p = 4; p <= 8; ++p)
-            for (int w = 4; w <= PK_MAX_WARPS; ++w) {
-                const int c = (nq + p * w - 1) / (p * w);
-                const long long cost = (long long)c * (32 * p * w + n);
-                if (best == 0 || cost < best) {
-                    best = cost;
-                    pt = p;
-                    nw = w;
-                    ctas = c;
-                }
-            }
+        const int pt = nq <= 4 ? 1 : (nq <= 8 ? 2 : 4);
+        return {pt, (nq + pt - 1) / pt, 1};
     }
+    PkPlan best = {};
+    long long least = 0;
+    for (int p = 4; p <= 8; ++p)
+        for (int w = 4; w <= PK_MAX_WARPS; ++w) {
+            const int c = (nq + p * w - 1) / (p * w);
+            const long long cost = (long long)c * (32 * p * w + n);
+            if (least == 0 || cost < least) {
+                least = cost;
+                best = {p, w, c};
+            }
+        }
+    return best;
+}
+
+// Packed pairs or tiles: both run at the FP64 pipe (600 and 610 GFMA/s counted
+// as here), so the fewer FP64 operations of a pole win. Packed pairs: every
+// lane of every warp load and the rows a CTA scales, those from its first
+// pair's on. Tiles: 64 x 64 (48 x 64 on the diagonal) and 64 columns to scale.
+// ms for 1000 poles, packed and tiled: 200 x 1000 energies 35.0, 61.4; 320 x
+// 400 37.6, 37.8; 384 x 300 40.3, 40.1; 448 x 200 36.7, 35.9; 500 x 160 37.1,
+// 37.4; 512 x 160 39.2, 37.2; 530 x 160 41.9, 46.7; 660 x 100 41.6, 43.3; 700
+// x 100 46.6, 43.3; 769 x 64 36.9, 38.5. Above PK_MAX_N one CTA of staged rows
+// fills an SM and the pipe idles at its barriers (833 x 64: 48.2, 44.4).
+constexpr int PK_MAX_N = 784;
+
+bool packed_wins(int n, const PkPlan &pl)
+{
+    if (n < 32) return true;
+    if (n > PK_MAX_N) return false;
+    const int span = 32 * pl.pt * pl.nw, t = (n + 63) / 64;
+    long long packed = 0;
+    for (int c = 0, i = 0; c < pl.ctas; ++c) {
+        while (i + 1 < n && tri_idx(i + 1, i + 1, n) <= c * span) ++i;
+        packed += span + n - i;
+    }
+    const long long tiled = (long long)t * (t - 1) / 2 * (64 * 64 + 64) + (long long)t * (48 * 64 + 64);
+    return 51 * packed <= 50 * tiled;
+}
+
+cudaError_t launch_packed_any(const PwDev &pw, const PkPlan &pl, const double *E, int nE, double *R, cudaStream_t s)
+{
+    const int n = pw.n, pt = pl.pt, nw = pl.nw, ctas = pl.ctas;
 #define RM_PK(P, K, D) launch_packed<P, K, D>(pw, E, nE, R, nw, ctas, s)
     if (n < 32) return pt == 1 ? RM_PK(1, 16, true) : (pt == 2 ? RM_PK(2, 16, true) : RM_PK(4, 16, true));
-    // poles per chunk: at most ~70 KB of shared memory, three CTAs per SM
-#define RM_PK_TK(P) (n <= 256 ? RM_PK(P, 16, false) : (n <= 512 ? RM_PK(P, 8, false) : RM_PK(P, 4, false)))
+    // poles per chunk: at most ~70 KB of shared memory (three CTAs per SM) up
+    // to 512 channels, two CTAs above (with 4 poles a chunk instead, 530 x 160
+    // took 47.5 ms, 41.9 so: a barrier comes too often)
+#define RM_PK_TK(P) (n <= 256 ? RM_PK(P, 16, false) : RM_PK(P, 8, false))
     switch (pt) {
     case 4: return RM_PK_TK(4);
     case 5: return RM_PK_TK(5);
@@ -163,7 +196,7 @@ constexpr int TB = 64;   // output tile
 constexpr int TK = 16;   // pole chunk
 constexpr int TT = 4;    // outputs per thread per dimension
 
-// n > PK_MAX_N: CTA per (energy, 64x64 upper tile); 256 threads x 4x4 outputs.
+// The rest: CTA per (energy, 64x64 upper tile); 256 threads x 4x4 outputs.
 // Off-diagonal tiles: thread (ty, tx) = (tid/16, tid%16) owns rows 4ty.., cols
 // 4tx... Diagonal tiles: the 32x32 quadrant below the diagonal is not needed,
 // so whole warps are assigned to the three upper quadrants (2 warps each) and
@@ -251,7 +284,8 @@ cudaError_t launch_form_r_fp64(const PwDev &pw, const double *E, int nE, double 
                                cudaStream_t s)
 {
     if (nE == 0) return cudaSuccess;
-    if (pw.n <= PK_MAX_N) return launch_packed_any(pw, E, nE, R, s);
+    const PkPlan pl = pk_plan(pw.n);
+    if (packed_wins(pw.n, pl)) return launch_packed_any(pw, pl, E, nE, R, s);
     const int t = (pw.n + TB - 1) / TB;
     dim3 grid(t, t, nE);
     form_r_tiled<<<grid, 256, 0, s>>>(pw, E, R);
