@@ -691,8 +691,20 @@ __device__ void chanfn_pair(const PwDev &pw, const double *__restrict__ E, int n
 // channels 270, 134, 106 us; 2000 of 4 906, 450, 395; 304 of 32 830, 432, 336;
 // 200 of 132 654, 500, 516; 1777 of 41 (z = 0) 2211, 252, 385; 4000 of 64 2.07,
 // 1.72, 2.03 ms. Up to XN_W8_PAIRS pairs leave the SMs room for eight lanes.
+// With the deep pairs in a list of their own and very many others, no single
+// pair decides, and lanes only cost: four take 1.5 times the FP64 instructions
+// that one thread takes. (Without a list the deepest pair is among them
+// and still lasts as long as the launch.) One thread against four
+// lanes, ms at z = 1 / 2 / 3: direct mode, 64 channels, 320 thousand pairs
+// 2.30, 2.31, 2.23 / 2.08, 2.24, 2.12; 448 thousand 2.91, 2.79, 2.62 / 2.88,
+// 2.79, 2.86; 640 thousand 3.83, 3.34, 3.27 / 3.85, 3.69, 3.70; 2.1 million
+// 7.42, 7.21, 7.17 / 10.4, 10.4, 10.2. The quantum-defect mode, whose series
+// one lane of a pair forms either way: 640 thousand 4.20, 4.18, 4.35 / 4.13,
+// 4.01, 4.07; 1.02 million 5.29, 5.45, 5.44 / 5.86, 5.92, 6.23. At z = 0 the
+// lanes win throughout (no tails; 1.28 million 5.64 / 4.10).
 constexpr int XN_BS = 128;                // threads per block
 constexpr long long XN_W8_PAIRS = 16384;
+constexpr long long XN_MAX_PAIRS = 7 << 16, XN_MAX_PAIRS_MQDT = 11 << 16;
 // z = 0: from this k a (kappa a) on, the fractions whose first numerator is
 // zero are not run for their tail, which converges there in well under
 // CF_MAXIT steps; nearer a threshold they are run as ever, and a tail that
@@ -1509,7 +1521,7 @@ cudaError_t launch_chanfn(const PwDev &pw, const double *E, int nE, const Opts &
 {
     const long long total = (long long)nE * pw.n;
     if (total == 0) return cudaSuccess;
-    if (no_tables(pw)) {
+    if (no_tables(pw) && (pw.z == 0.0 || !deep_ws || total <= (mqdt ? XN_MAX_PAIRS_MQDT : XN_MAX_PAIRS))) {
         if (total <= XN_W8_PAIRS) launch_xn<8>(pw, E, nE, o, mqdt, cf, status, deep_ws, nullptr, total, s);
         else launch_xn<4>(pw, E, nE, o, mqdt, cf, status, deep_ws, nullptr, total, s);
         return cudaGetLastError();
