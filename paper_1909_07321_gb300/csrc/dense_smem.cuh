@@ -20,6 +20,12 @@ constexpr int SOLVE_SMALL_MAXN = 96;
 constexpr int NT = 256;
 
 
+// Right-hand column that pair of lanes `pair` reads, one pair a column. Pairs
+// past the last column, which only take part in their warp's exchanges, read
+// that one: it belongs to their own warp (no pair of a warp without a column
+// gets here), so that no other warp writes it meanwhile.
+__host__ __device__ inline int pair_column(int pair, int n_rhs) { return pair < n_rhs ? pair : n_rhs - 1; }
+
 struct ElimShared {
     int piv;
     int bad;

@@ -303,7 +303,7 @@ __device__ void cblock_backsub(double2 *M, int ld, int rows, int rhs0, int n_rhs
         // whole warps take part in the exchanges
         if (q0 + ((threadIdx.x & ~31) >> 1) >= n_rhs) break;
         const bool on = qq < n_rhs;
-        const int cq = rhs0 + (on ? qq : 0);
+        const int cq = rhs0 + pair_column(qq, n_rhs);
         for (int t = rows - 1; t >= 0; --t) {
             const double2 s0 = M[t * ld + cq];
             double s = im ? s0.y : s0.x;
