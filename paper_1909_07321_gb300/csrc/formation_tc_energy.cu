@@ -29,6 +29,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "float_bits.cuh"
 #include "tc_sm103.cuh"
 
 namespace rmgb {
@@ -407,50 +408,6 @@ __global__ void pe_d32_kernel(PwDev pw, const double *__restrict__ E, int nE, do
         while (k1 < pw.N && pw.Ek[k1] < x + delta) ++k1;
         np_range[e] = make_int2(lo, k1);
     }
-}
-
-// s = v[0] + v[1] + ... (FP64, in this order) of n <= 8 floats. The FP64 unit
-// does 2 additions or conversions per clock and SM, and the 17 of an entry of 8
-// segments held this kernel at 5.3 ms for 256 energies of 1000 channels
-// (2.05 with this; the partials' traffic is 1.0). While the exponents of the
-// nonzero values lie within 26 of one another, every partial sum is a multiple
-// of the smallest unit below 2^53 of it, so the FP64 sum is exact: the
-// mantissas are then summed as integers and converted once. Otherwise (and for
-// subnormal or non-finite values) the plain sum is taken.
-__device__ __forceinline__ double pe_sum(const float (&v)[8], int n)
-{
-    int lo = 255, hi = 0;
-    bool odd = false;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        if (q >= n) continue;
-        const uint32_t u = __float_as_uint(v[q]) & 0x7fffffffu;
-        const int e = (int)(u >> 23);
-        odd = odd || e == 255 || (e == 0 && u != 0u);
-        if (u != 0u) {
-            lo = min(lo, e);
-            hi = max(hi, e);
-        }
-    }
-    if (odd || hi - lo > 26) {
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q < n) s += (double)v[q];
-        return s;
-    }
-    long long sum = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        if (q >= n) continue;
-        const uint32_t u = __float_as_uint(v[q]);
-        const int e = (int)((u >> 23) & 255u);
-        const int m = e ? (int)((u & 0x7fffffu) | 0x800000u) : 0;
-        sum += (long long)((u >> 31) ? -m : m) * (long long)(1 << (e ? e - lo : 0));
-    }
-    if (sum == 0) return 0.0;
-    const double d = (double)sum;   // exact
-    return __hiloint2double(__double2hiint(d) + ((lo - 150) << 20), __double2loint(d));
 }
 
 // R_ij for j >= i = (1/2a) [sum over segments of the FP32 partials (in FP64,

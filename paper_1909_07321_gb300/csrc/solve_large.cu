@@ -38,6 +38,7 @@
 #include <algorithm>
 
 #include "dense_global_f32.cuh"
+#include "float_bits.cuh"
 #include "rm_internal.cuh"
 
 namespace rmgb {
@@ -1017,20 +1018,6 @@ __global__ void omega_kernel(PwDev pw, const double *__restrict__ E, int nE,
 }
 
 // ---- FP32 path ---------------------------------------------------------------
-
-// (float)v without the FP64 unit: round to nearest even on the bits where the
-// result is a normal float, the conversion instruction elsewhere.
-__device__ __forceinline__ float to_float(double v)
-{
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const unsigned mh = hi & 0x7fffffffu;
-    // 2^-126 <= |v| < 2^127
-    if (mh - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)v;
-    const unsigned t = ((mh - 0x38000000u) << 3) | (lo >> 29);   // exponent and 23 bits
-    const unsigned rest = lo << 3;                                // the bits below
-    const unsigned up = (rest > 0x80000000u || (rest == 0x80000000u && (t & 1u))) ? 1u : 0u;
-    return __uint_as_float((hi & 0x80000000u) | (t + up));
-}
 
 // [A | 0 | B] in FP32: A = diag(Ghat) - R diag(a Ghat' - b Ghat), B as in
 // assemble_kernel, right-hand sides from column rhs0(n), zero padding. A CTA
