@@ -558,9 +558,11 @@ def _dist(x):
 
 
 def _pe_tiles(n):
-    """Tiles of 128 rows x 256 columns holding some (i <= j) of an n x n matrix."""
+    """Tiles of 128 rows x 256 columns holding some (i <= j) of an n x n matrix, less the halves that the kernel
+    leaves out: the left one where the rows start at its end, the right one where it lies past the last column."""
     n_ib, n_jb = -(-n // 128), -(-n // 256)
-    return sum(min(n_ib, 2 * jb + 2) for jb in range(n_jb))
+    return sum(1.0 - 0.5 * (ib >= 2 * jb + 1) - 0.5 * (n - 256 * jb <= 128)
+               for jb in range(n_jb) for ib in range(min(n_ib, 2 * jb + 2)))
 
 
 def run_wide(args, prec, sp, stream, flush, peaks, peak_src):
@@ -611,7 +613,7 @@ def run_wide(args, prec, sp, stream, flush, peaks, peak_src):
             "executed_frac": 3.0 * alg * _pe_tiles(n) * 128 * 256 / (n * (n + 1) / 2) / tpk,
             "traffic": None, "kernel": "form_r_pe_kernel (%s, one GEMM per energy)" % args.precision,
             "note": ("algorithmic n(n+1)N flops per energy; issued x3 (hi/lo products); executed "
-                     "counts the tiles of 128 x 256 that cover the upper triangle"),
+                     "counts the tiles of 128 x 256 that cover the upper triangle, less the halves left out"),
             "peak_source": ("bf16 dense burst, %s" % peak_src) if prec == 2 else
             ("tf32 = bf16 dense burst (%s) x nominal ratio 1/2" % peak_src)}})
     return out
