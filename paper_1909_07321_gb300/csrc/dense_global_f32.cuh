@@ -1,8 +1,8 @@
 // FP32 dense kernels of the global-memory solver's mixed-precision path
 // (rm_opts.solve_precision = RM_FP32, channel counts above the shared-memory
-// solver's limit). One CTA (256 threads for the narrower systems, so that two
-// share an SM, 512 for the wider ones) works on one energy's matrices in
-// global memory:
+// solver's limit). One CTA works on one energy's matrices in global memory: 128
+// or 256 threads for the narrower systems, so that several share an SM, 512 for
+// the wider ones (launch_lu32_any and launch_zsweep_any, solve_large.cu):
 //
 //   lu32_factor_solve   [A | B] -> solves A X = B for the trailing rows of X
 //                       (the matching system, Section "Overview", Eq. match):
@@ -15,9 +15,10 @@
 //                       U12 = L11^{-1} A12 is solved one column per thread;
 //                       the trailing matrix takes the rank-PB update
 //                       A22 -= L21 U12 in strips of 128 columns with 4 x 8
-//                       register tiles per thread, packed FMAs (the U12 strips
-//                       copied asynchronously into two shared buffers in
-//                       turn). Back-substitution of the
+//                       or (two panel rows a thread) 8 x 8 register tiles per
+//                       thread, packed FMAs (the U12 strips copied
+//                       asynchronously into two shared buffers in turn).
+//                       Back-substitution of the
 //                       requested rows runs in the same blocked form, upwards.
 //   zsweep_invert       Z <- -Z^{-1} for a complex symmetric Z whose
 //                       Hermitian part is positive definite (Z = 1 - iK, the
@@ -36,10 +37,12 @@
 //                       takes the entry (min(i, j), max(i, j)).
 //
 // At 1000 channels both stream their trailing matrix through HBM once per
-// panel (152 CTAs hold 1.2 GB) and are bound by that; below about 300 they
-// were bound by the latency of the panel's columns, which the registers and
-// the second CTA per SM take away. ms for 304 or more systems filling the GPU,
-// before and after: LU of 110 unknowns (1216 systems) 1.61 -> 0.46, 203 (912)
+// panel (152 CTAs hold 1.2 GB), but what their inner loops wait for is shared
+// memory, from which every FMA's operands come (64 energies: L1 and shared
+// memory 48% and 75% busy in LU and sweep, FMA pipe 46% and 48%, DRAM 10% and
+// 7%); below about 300 they were bound by the latency of the panel's columns,
+// which the registers and the second CTA per SM take away. ms for 304 or more
+// systems filling the GPU, before and after: LU of 110 unknowns (1216 systems) 1.61 -> 0.46, 203 (912)
 // 2.85 -> 1.11, 431 (456) 5.37 -> 3.44, 1000 (304, 600 right-hand sides) 22.1
 // -> 19.1; sweep of 80 (1216) 0.63 -> 0.39, 150 (912) 1.38 -> 1.00, 300 (456)
 // 2.79 -> 2.30, 600 (304) 11.5 -> 11.0. Every entry keeps its chain of FMAs,

@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(NTH, 2) lu64_kernel(const LuJob *__restrict__ 
 {
     extern __shared__ double sm64[];
     constexpr int NW = NTH / 32;
-    __shared__ double slots[NW][PNB + 2];   // a warp's candidate: its row, key, row number
+    __shared__ double slots[NW][PNB + 2];   // the row of a warp's candidate (key and number: red_k, red_i)
     __shared__ unsigned long long red_k[NW];
     __shared__ int red_i[NW];
     __shared__ int s_bad, s_moves, s_piv, s_win, mv_dst[PNB], mv_src[PNB];

@@ -394,7 +394,10 @@ class Context:
 
     By default the context enqueues on torch's current stream of `device`, so
     its work is ordered with the torch operations that fill its inputs and
-    read its outputs."""
+    read its outputs. With stream=0 it has a stream of its own, which torch's
+    operations are not ordered with; there, unless lane_stream() has given the
+    stream out, collision_strengths() copies rows into page-locked memory
+    while later ones are still being solved (include/rmgb.h)."""
 
     def __init__(self, precision=0, stream=None, mem_budget=0, device=0, **kw):
         o = rm_default_opts()
